@@ -163,6 +163,8 @@ def schedule_name(lb, g, scheme):
             return "st quad (128-bit words, f32x2), four cells per thread"
         return "st pair (f32x2), two cells per thread"
     k, c = g.fv_schedule()
+    if k == lb.LB_FV_TILE and c == 2:
+        return "fv two launches (predictor, corrector), no tile"
     if k == lb.LB_FV_TILE:
         return "fv tile %s (halo 4)" % {0: "32x16", 16: "16x16", 8: "16x8"}[c]
     if k == lb.LB_FV_SPLIT:

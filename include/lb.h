@@ -133,8 +133,8 @@ lb_status lb_init(lb_grid* grid, const lb_params* params, const lb_init_desc* in
  * interpolated to the faces by QUICK (Sec. II B 3), walls use the double
  * reflection of Sec. II B 5 on h (thermal field: anti-reflection through
  * T_wall), the predictor f~* is Eq. (semi) and the corrector averages the
- * two flux divergences.  One fused kernel launch per step (long runs replay
- * the launches as a CUDA graph: lb_set_graph_steps).
+ * two flux divergences.  One fused kernel launch per step, or two (long runs
+ * replay the launches as a CUDA graph: lb_set_graph_steps).
  * LB_ERR_STATE if the grid has no parameters or is poisoned. */
 lb_status lb_step_fv(lb_grid* grid, int nsteps);
 
@@ -165,7 +165,10 @@ lb_status lb_get_graph_steps(lb_grid* grid, int* n, unsigned long long* replays)
 /* Kernel schedule of lb_step_fv.  All kernels compute the same step
  * (Eq. (semi-heun)); they differ only in how the grid is cut into CTAs:
  *   LB_FV_TILE:  32 x 16 tiles with a 4-cell halo in both axes, three
- *                shared-memory regions per tile;
+ *                shared-memory regions per tile; chunk 2: no tiles, the
+ *                predictor and the corrector as two launches over the whole
+ *                grid, through three library-owned fields allocated on first
+ *                use (where that fails the 32 x 16 tiles run instead);
  *   LB_FV_MARCH: strips of 120 columns (56 for FP64 thermal) that march up
  *                `chunk` rows each, halo only in x;
  *   LB_FV_PAIR:  the marching strips with two columns per thread and packed
@@ -182,7 +185,8 @@ lb_status lb_get_graph_steps(lb_grid* grid, int* n, unsigned long long* replays)
  *                f~ + Coll - dt/2 A[h^n] pass through two library-owned FP32
  *                buffers allocated on first use (same restrictions as
  *                LB_FV_PAIR); chunk 0 = 32 x 16, 16 = 16 x 16.
- * LB_FV_AUTO picks by grid size.  For the marching kernels chunk = 0 lets
+ * LB_FV_AUTO picks by grid size and storage (on FP64 grids and on small ones
+ * the two launches of LB_FV_TILE, chunk 2).  For the marching kernels chunk = 0 lets
  * the library size the chunks to fill the GPU; for LB_FV_TILE chunk picks
  * the tile: 0 = 32 x 16, 16 = 16 x 16, 8 = 16 x 8 (smaller tiles recompute
  * more halo but suit small, latency-bound grids).  LB_ERR_ARG on an unknown
@@ -220,7 +224,7 @@ lb_status lb_set_fv_scheme(lb_grid* grid, int scheme);
 lb_status lb_get_fv_scheme(lb_grid* grid, int* scheme);
 
 /* Autotuner: times `steps` FV steps for each candidate schedule (the three
- * tile shapes; march and pair with several chunk lengths; the paired tiles
+ * tile shapes; the two-launch step where its fields can be allocated; march and pair with several chunk lengths; the paired tiles
  * and the split schedule where they apply) on the grid's current state,
  * restores the state after each candidate, and keeps the fastest.
  * Synchronous; uses a temporary copy of the populations (and allocates the

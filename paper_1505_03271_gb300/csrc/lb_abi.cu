@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "lb_grid.cuh"
+#include "lb_phase.cuh"
 
 using namespace lbgb;
 
@@ -76,7 +77,7 @@ namespace {
 void release(lb_grid* G) {
     void* ptrs[] = {G->f[0], G->f[1], G->g[0], G->g[1], G->mx, G->my, G->dxv, G->dyv, G->xc,
                     G->yc, G->toff, G->toff_r, G->roff, G->roff_r, G->dref_r, G->rowtab, G->coltab, G->fields,
-                    G->partial, G->red, G->xh, G->xfc};
+                    G->partial, G->red, G->xh, G->xfc, G->fold[0], G->fold[1], G->phase};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (G->cap) cudaStreamDestroy(G->cap);
@@ -190,6 +191,66 @@ cudaError_t launch_fv_step(lb_grid* G) {
                                                  G->stream);
     if (k == LB_FV_MARCH) return launch_fv_march(G->prec, th, &A, resolved_chunk(G), G->stream);
     return launch_fv(G->prec, th, &A, G->fv_kernel == LB_FV_TILE ? G->fv_chunk : 0, G->stream);
+}
+
+// Whether lb_step_fv runs the two-launch step of k_fv_phase.cu: FP64 grids
+// of every size (the fused kernels recompute on the scarce FP64 pipe), and
+// FP32-math grids up to 128 cells per SM (thermal: 64), where the fused tile
+// leaves most SMs idle: 128 x 128 FP32 takes 4.4 us a step against 6.1,
+// 192 x 192 8.1 against 6.3; thermal 96 x 96 4.9 against 9.1, 128 x 128 8.9
+// against 9.1.  Its kernels address a pair of planes with 32-bit offsets.
+bool phase_applies(const lb_grid* G) {
+    if (G->fv_scheme != LB_FV_HEUN || has_density_axis(G)) return false;
+    const bool f64 = G->prec == Prec::F64;
+    if (3ULL * G->plane * (f64 ? 8 : 4) >= 1ULL << 32) return false;
+    if (G->fv_kernel != LB_FV_AUTO) return G->fv_kernel == LB_FV_TILE && G->fv_chunk == 2;
+    return f64 || (G->d.thermal ? 2LL : 1LL) * G->nx * G->ny <= 128LL * G->sms;
+}
+
+// The two-launch step's fields, allocated on first use; false where that is
+// not possible (no memory, or a stream capture in progress forbids it): the
+// step then takes the fused kernels.
+bool ensure_phase(lb_grid* G) {
+    if (G->phase) return true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(G->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    const size_t rs = G->prec == Prec::F64 ? 8 : 4;
+    if (cudaMalloc(&G->phase, 3 * rs * (G->d.thermal ? 18 : 9) * (size_t)G->plane) != cudaSuccess) {
+        cudaGetLastError();
+        G->phase = nullptr;
+        return false;
+    }
+    return true;
+}
+
+// start: h of the present state (before the first step of a call); else one step
+template <typename R>
+cudaError_t launch_phase(lb_grid* G, bool start) {
+    const size_t set = (G->d.thermal ? 18 : 9) * (size_t)G->plane;
+    R* w = static_cast<R*>(G->phase);
+    PhaseArgs<R> P{};
+    P.s = step_args<R>(G, G->p.dt);
+    P.h = w;
+    P.hs = w + set;
+    P.b = w + 2 * set;
+    P.foldx = static_cast<const R*>(G->fold[0]);
+    P.foldy = static_cast<const R*>(G->fold[1]);
+    const double dt = G->p.dt;
+    for (int q = 0; q < 2; ++q) {
+        const double k = dt / (2.0 * (q ? G->p.tau_g : G->p.tau) + dt);  // omh, omgh
+        P.k[q] = (R)k;
+        P.kh[q] = (R)(0.5 * k);
+    }
+    P.ctx = (R)(3.0 * 0.5 * dt * (1.0 - dt / (2.0 * G->p.tau + dt)) * G->p.ax);
+
+    return launch_fv_phase(G->prec, G->d.thermal != 0, &P, start, G->sms, G->stream);
+}
+
+cudaError_t launch_phase(lb_grid* G, bool start) {
+    return G->prec == Prec::F64 ? launch_phase<double>(G, start) : launch_phase<float>(G, start);
 }
 
 lb_status upload(void** dst, const std::vector<double>& v, bool as_float) {
@@ -402,6 +463,8 @@ lb_status lb_create_grid(const lb_grid_desc* d, lb_grid** out) {
     alloc((void**)&G->red, sizeof(double) * kRed);
     if (st == LB_OK) st = upload(&G->mx, G->ax.metric(), as_float);
     if (st == LB_OK) st = upload(&G->my, G->ay.metric(), as_float);
+    if (st == LB_OK) st = upload(&G->fold[0], G->ax.cell_weights(as_float), as_float);
+    if (st == LB_OK) st = upload(&G->fold[1], G->ay.cell_weights(as_float), as_float);
     if (st == LB_OK) st = upload((void**)&G->dxv, G->ax.d, false);
     if (st == LB_OK) st = upload((void**)&G->dyv, G->ay.d, false);
     if (st == LB_OK) st = upload((void**)&G->xc, G->ax.c, false);
@@ -578,6 +641,10 @@ lb_status lb_step_fv(lb_grid* G, int nsteps) {
     if (s != LB_OK) return s;
     if (nsteps < 0) return fail(LB_ERR_ARG, "nsteps must be >= 0");
     DeviceGuard dg(G->device);
+    if (nsteps > 0 && phase_applies(G) && ensure_phase(G)) {
+        CK(launch_phase(G, true));
+        return run_steps(G, nsteps, [G] { return launch_phase(G, false); });
+    }
     return run_steps(G, nsteps,
                      [G] { return G->prec == Prec::F64 ? launch_fv_step<double>(G) : launch_fv_step<float>(G); });
 }
@@ -600,8 +667,8 @@ lb_status lb_set_fv_schedule(lb_grid* G, int kernel, int chunk) {
     if (!G) return fail(LB_ERR_ARG, "grid is NULL");
     if (kernel < LB_FV_AUTO || kernel > LB_FV_SPLIT) return fail(LB_ERR_ARG, "unknown FV kernel %d", kernel);
     if (chunk < 0) return fail(LB_ERR_ARG, "chunk must be >= 0");
-    if (kernel == LB_FV_TILE && chunk != 0 && chunk != 8 && chunk != 16)
-        return fail(LB_ERR_ARG, "tile shape must be 0 (32 x 16), 16 (16 x 16) or 8 (16 x 8)");
+    if (kernel == LB_FV_TILE && chunk != 0 && chunk != 8 && chunk != 16 && chunk != 2)
+        return fail(LB_ERR_ARG, "tile shape must be 0 (32 x 16), 16 (16 x 16), 8 (16 x 8) or 2 (two launches, no tile)");
     if (kernel == LB_FV_PTILE && chunk != 0 && chunk != 14 && chunk != 16 && chunk != 512 && chunk != 526)
         return fail(LB_ERR_ARG, "paired tile shape must be 0 (32 x 16), 14 (32 x 14), 16 (16 x 16), 512 (32 x 16, "
                                 "512 threads) or 526 (32 x 14, 512 threads)");
@@ -643,6 +710,11 @@ lb_status lb_get_fv_scheme(lb_grid* G, int* scheme) {
 
 lb_status lb_get_fv_schedule(lb_grid* G, int* kernel, int* chunk) {
     if (!G) return fail(LB_ERR_ARG, "grid is NULL");
+    if (phase_applies(G)) {
+        if (kernel) *kernel = LB_FV_TILE;
+        if (chunk) *chunk = 2;
+        return LB_OK;
+    }
     if (kernel) *kernel = resolved_kernel(G);
     if (chunk) {
         const int k = resolved_kernel(G);
@@ -680,6 +752,8 @@ lb_status lb_autotune_fv(lb_grid* G, int steps) {
             cands.push_back({LB_FV_SPLIT, 16});
         }
     }
+    const bool had_phase = G->phase != nullptr;
+    cands.push_back({LB_FV_TILE, 2});
     for (int kern : {(int)LB_FV_MARCH, (int)LB_FV_PAIR}) {
         if (kern == LB_FV_PAIR && !pair_ok(G)) continue;
         G->fv_kernel = kern;
@@ -698,12 +772,19 @@ lb_status lb_autotune_fv(lb_grid* G, int steps) {
         G->fv_kernel = c.first;
         G->fv_chunk = c.second;
         G->cur = cur0;
+        const bool phase = c == std::make_pair((int)LB_FV_TILE, 2);
+        if (phase && !(phase_applies(G) && ensure_phase(G))) continue;
+        auto one = [&] {
+            return phase ? launch_phase(G, false)
+                         : G->prec == Prec::F64 ? launch_fv_step<double>(G) : launch_fv_step<float>(G);
+        };
         // warm-up step, then the timed ones
-        cudaError_t e = G->prec == Prec::F64 ? launch_fv_step<double>(G) : launch_fv_step<float>(G);
+        cudaError_t e = phase ? launch_phase(G, true) : cudaSuccess;
+        if (e == cudaSuccess) e = one();
         G->cur ^= 1;
         cudaEventRecord(e0, G->stream);
         for (int k = 0; k < steps && e == cudaSuccess; ++k) {
-            e = G->prec == Prec::F64 ? launch_fv_step<double>(G) : launch_fv_step<float>(G);
+            e = one();
             G->cur ^= 1;
         }
         cudaEventRecord(e1, G->stream);
@@ -728,6 +809,10 @@ lb_status lb_autotune_fv(lb_grid* G, int steps) {
     cudaEventDestroy(e1);
     cudaFree(sf);
     if (sg) cudaFree(sg);
+    if (!had_phase && G->phase && (st != LB_OK || pick != std::make_pair((int)LB_FV_TILE, 2))) {
+        cudaFree(G->phase);
+        G->phase = nullptr;
+    }
     if (st != LB_OK) {
         G->fv_kernel = k0;
         G->fv_chunk = c0;

@@ -68,6 +68,32 @@ struct Axis {
         for (int i = 0; i < n; ++i) m[6 * (n + 1) + i] = 1.0 / d[i];
         return m;
     }
+    // Per cell, for c > 0 and then for c < 0, the two-launch step's weights
+    // of c (Phi_e - Phi_w) / dx.  FP64: K[4] with the sum K_s h_s over the
+    // nodes (from -2 for c > 0, from -1 for c < 0).  FP32: the west and the
+    // east face's three weights, c / dx and a pad.
+    std::vector<double> cell_weights(bool f32) const {
+        const int m = f32 ? 8 : 4;
+        std::vector<double> t(2 * (size_t)m * n, 0.0);
+        for (int i = 0; i < n; ++i)
+            for (int sg = 0; sg < 2; ++sg) {
+                double w[3], e[3];
+                quick(sg ? i - 1 : i - 2, i, w);
+                quick(sg ? i : i - 1, i + 1, e);
+                const double s = (sg ? -1.0 : 1.0) / d[i];
+                double* k = &t[(size_t)m * (2 * i + sg)];
+                if (f32) {
+                    for (int r = 0; r < 3; ++r) k[r] = w[r], k[3 + r] = e[r];
+                    k[6] = s;
+                } else {
+                    k[0] = -w[0] * s;
+                    k[1] = (e[0] - w[1]) * s;
+                    k[2] = (e[1] - w[2]) * s;
+                    k[3] = e[2] * s;
+                }
+            }
+        return t;
+    }
 };
 
 inline Axis make_axis(int n, double L, int sp, double st, int bc) {
@@ -127,6 +153,8 @@ struct lb_grid {
     float* coltab = nullptr;    // [nx][20] x weights of a column pair and its 1/dx (paired tile kernel)
     float* xh = nullptr;        // split schedule: h*, [NQ][ny][pitch] FP32 (allocated on first use)
     float* xfc = nullptr;       // split schedule: f~ + Coll - dt/2 A[h^n]
+    void* fold[2] = {nullptr, nullptr};  // Axis::cell_weights of x and y, compute precision
+    void* phase = nullptr;      // two-launch step: h, h*, b, each [NQ][ny][pitch] (allocated on first use)
     double* fields = nullptr;   // [4][ny][nx] staging for init/moments
     double* partial = nullptr;  // reduction partials
     double* red = nullptr;      // reduction totals

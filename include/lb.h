@@ -171,9 +171,11 @@ lb_status lb_get_graph_steps(lb_grid* grid, int* n, unsigned long long* replays)
  *                use (where that fails the 32 x 16 tiles run instead);
  *   LB_FV_MARCH: strips of 120 columns (56 for FP64 thermal) that march up
  *                `chunk` rows each, halo only in x;
- *   LB_FV_PAIR:  the marching strips with two columns per thread and packed
- *                FP32 pair arithmetic; FP32/FP16/BF16 storage and x-periodic
- *                grids only (LB_ERR_ARG otherwise);
+ *   LB_FV_PAIR:  strips that march up `chunk` rows (rounded up to a multiple
+ *                of 4) in blocks of four, collision, predictor and corrector
+ *                on warps of their own, in packed FP32 pair arithmetic;
+ *                FP32/FP16/BF16 storage and x-periodic grids only
+ *                (LB_ERR_ARG otherwise);
  *   LB_FV_PTILE: the tiles with two columns per thread-cell and packed FP32
  *                pair arithmetic (same restrictions); chunk 0 = 32 x 16,
  *                14 = 32 x 14, 16 = 16 x 16, 512 = 32 x 16 with 512 threads

@@ -5,12 +5,10 @@
 //              h*, and b = f~ + Coll - dt/2 A[h^n]
 //   corrector  A[h*] -> f~^(n+1) = b - dt/2 A[h*], its moments and h^(n+1),
 //              which the next step's predictor reads
-// One launch before the first step of a call forms h^n and f~ + Coll.  Since
-// om = 2 omh and cf = 2 hF, the small change t = h - f~ gives both: h = f~ + t
-// and f~ + Coll = f~ + 2 t, one relaxation instead of two, and only t is
-// rounded on the way (f~ + Coll as 2 h - f~ would double the rounding of h,
-// which shows: 2.3 times the FP32 error of a slowly driven channel).  b holds
-// f~ + Coll between the steps, so the state is written but never read.
+// One launch before the first step of a call forms h^n and f~ + Coll.  FP64
+// forms both from one relaxation: om = 2 omh and cf = 2 hF, so with the change
+// t = h - f~, f~ + Coll = f~ + 2 t.  FP32 rounds as the paired kernels do,
+// whose results it reproduces bit for bit, and takes two.
 // b holds f~ + Coll between the steps, so the state is written but not read.
 // h, h* and b are fields of the compute type in memory: a step streams eight
 // values per population and cell instead of two.
@@ -25,6 +23,7 @@
 // FP64 step, fused tile -> this: 1 x 64 132 -> 7.4 us, 64 x 64 132 -> 8.7 us,
 // 1024 x 1024 2011 -> 649 us (0.52 -> 1.62 GLUPS).  FP32: 64 x 64 6.1 -> 3.4
 // us, thermal 64 x 64 (16-bit) 9.0 -> 4.0 us.
+#include "lb_pair.cuh"
 #include "lb_phase.cuh"
 
 namespace lbgb {
@@ -158,22 +157,36 @@ __device__ __forceinline__ void advect_sites(const R* H, const Site<R>& s, const
 template <typename R, bool TH, bool FC>
 __device__ __forceinline__ void store_h(const R* d, const R* e, const PhaseArgs<R>& P, int y, R* H, unsigned c) {
     const StepArgs<R>& A = P.s;
-    CellMom<R, TH> m;
-    m.build(d, e, A, TH ? A.roff[y] : R(0), TH ? A.toff[y] : R(0));
     const unsigned o = c * (unsigned)sizeof(R);
-    R t[Q];
-    m.change_f(d, P, t);
-#pragma unroll
-    for (int a = 0; a < Q; ++a) {
-        ref<R>(H + a * A.plane, o) = d[a] + t[a];
-        if constexpr (FC) ref<R>(P.b + a * A.plane, o) = d[a] + R(2) * t[a];
-    }
-    if constexpr (TH) {
-        m.change_g(e, P, t);
+    if constexpr (sizeof(R) == 8) {
+        CellMom<TH> m;
+        m.build(d, e, A, TH ? A.roff[y] : R(0), TH ? A.toff[y] : R(0));
+        R t[Q];
+        m.change_f(d, P, t);
 #pragma unroll
         for (int a = 0; a < Q; ++a) {
-            ref<R>(H + (Q + a) * A.plane, o) = e[a] + t[a];
-            if constexpr (FC) ref<R>(P.b + (Q + a) * A.plane, o) = e[a] + R(2) * t[a];
+            ref<R>(H + a * A.plane, o) = d[a] + t[a];
+            if constexpr (FC) ref<R>(P.b + a * A.plane, o) = d[a] + R(2) * t[a];
+        }
+        if constexpr (TH) {
+            m.change_g(e, P, t);
+#pragma unroll
+            for (int a = 0; a < Q; ++a) {
+                ref<R>(H + (Q + a) * A.plane, o) = e[a] + t[a];
+                if constexpr (FC) ref<R>(P.b + (Q + a) * A.plane, o) = e[a] + R(2) * t[a];
+            }
+        }
+    } else {
+        pairmath::LaneMom<TH> m;
+        m.build(d, e, A, TH ? A.roff[y] : 0.0f, TH ? A.toff[y] : 0.0f);
+#pragma unroll
+        for (int a = 0; a < Q; ++a) {
+            ref<R>(H + a * A.plane, o) = m.one_f(a, d[a], A, A.omh, A.hF);
+            if constexpr (FC) ref<R>(P.b + a * A.plane, o) = m.one_f(a, d[a], A, A.om, A.cf);
+            if constexpr (TH) {
+                ref<R>(H + (Q + a) * A.plane, o) = m.one_g(a, e[a], A.omgh);
+                if constexpr (FC) ref<R>(P.b + (Q + a) * A.plane, o) = m.one_g(a, e[a], A.omg);
+            }
         }
     }
 }
@@ -259,24 +272,28 @@ __global__ void __launch_bounds__(128) k_phase_correct(const PhaseArgs<R> P) {
 // whose warps run alone on their SM, is not bound by one long dependent
 // stream.
 //
-// QUICK divergence of one line of one population.  FP32 differences the two
-// face values, which the neighbours form from the same nodes and weights, so
-// a face's rounding cancels between its two cells: with folded weights 200
-// FP32 steps of a 64 x 48 vortex ended with four times the velocity error
-// (1.5e-5 against 3.6e-6, before the collision kept momentum exactly).
-// FP64 folds: half the instructions, and no error that shows.
+// One axis of one population.  FP64 takes the folded weights: half the
+// instructions of two face values.  FP32 forms the faces, in the order of
+// operations of the paired kernels, whose results it then reproduces bit for
+// bit (y: v + c (Phi_n - Phi_s) / dy; x: c (Phi_e - Phi_w) / dx).
 template <typename R>
 struct Quick {
-    float4 p, q;  // west face's weights and the east face's first; its others and c / dx
+    float4 p, q;  // west face's weights and the east face's first; its others and 1 / dx
     __device__ __forceinline__ void load(const float* t, int i, int v) {
         const float4* c = reinterpret_cast<const float4*>(t) + 4 * i + (v > 0 ? 0 : 2);
         p = __ldg(c);
         q = __ldg(c + 1);
     }
-    __device__ __forceinline__ float div(const float* h) const {
-        const float pw = p.x * h[0] + p.y * h[1] + p.z * h[2];
-        const float pe = p.w * h[1] + q.x * h[2] + q.y * h[3];
-        return (pe - pw) * q.z;
+    __device__ __forceinline__ float x(const float* h, int v) const {
+        const float w = __fmaf_rn(p.z, h[2], __fmaf_rn(p.x, h[0], __fmul_rn(p.y, h[1])));
+        const float e = __fmaf_rn(q.y, h[3], __fmaf_rn(p.w, h[1], __fmul_rn(q.x, h[2])));
+        const float d = __fmul_rn(e - w, q.z);
+        return v > 0 ? d : -d;
+    }
+    __device__ __forceinline__ float y(const float* h, int v, float sum) const {
+        const float s = __fmaf_rn(p.x, h[0], __fmaf_rn(p.y, h[1], __fmul_rn(p.z, h[2])));
+        const float n = __fmaf_rn(p.w, h[1], __fmaf_rn(q.x, h[2], __fmul_rn(q.y, h[3])));
+        return v > 0 ? __fmaf_rn(n - s, q.z, sum) : sum - __fmul_rn(n - s, q.z);
     }
 };
 template <>
@@ -286,9 +303,10 @@ struct Quick<double> {
 #pragma unroll
         for (int s = 0; s < 4; ++s) k[s] = __ldg(t + 8 * i + (v > 0 ? 0 : 4) + s);
     }
-    __device__ __forceinline__ double div(const double* h) const {
+    __device__ __forceinline__ double x(const double* h, int) const {
         return k[0] * h[0] + k[1] * h[1] + k[2] * h[2] + k[3] * h[3];
     }
+    __device__ __forceinline__ double y(const double* h, int v, double sum) const { return sum + x(h, v); }
 };
 
 __device__ __forceinline__ int vel(unsigned packed, int a) { return (int)((packed >> (2 * a)) & 3u) - 1; }
@@ -296,12 +314,23 @@ __host__ __device__ constexpr unsigned pack_vel(int axis, int a = 0) {
     return a == Q ? 0u : ((unsigned)((axis ? cy(a) : cx(a)) + 1) << (2 * a)) | pack_vel(axis, a + 1);
 }
 
+__device__ __forceinline__ double mad(double a, double b, double c) { return a * b + c; }
+__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+// the base state's flux divergence c_y w A[ref], as the paired kernels add it
+__device__ __forceinline__ double add_base(double v, double w, double r) { return v + w * r; }
+__device__ __forceinline__ float add_base(float v, float w, float r) { return v + __fmul_rn(w, r); }
+
+template <typename R, bool TH> struct MomOf;
+template <bool TH> struct MomOf<double, TH> { using T = CellMom<TH>; };
+template <bool TH> struct MomOf<float, TH> { using T = pairmath::LaneMom<TH>; };
+
 template <typename R, typename S, bool TH, bool CORR, int CELLS>
 __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const PhaseArgs<R> P) {
     constexpr int NQ = TH ? 2 * Q : Q;
-    constexpr int NM = TH ? 11 : 8;
+    constexpr int NM = TH ? 9 : 7;
     __shared__ R sd[NQ][CELLS];
-    __shared__ R sm[NM][CELLS];  // rp, rho, 3 ux, 3 uy, rho ux, rho uy, C0, 3 hF a_y; Td, T, C0 of g
+    // rp, rho, 3 ux, 3 uy; -1.5 u.u, -3 u.a, a_y (FP64: C0 of f and of g, 3 hF a_y); Td, T
+    __shared__ R sm[NM][CELLS];
     const StepArgs<R>& A = P.s;
     const int lane = threadIdx.x % CELLS, i = threadIdx.x / CELLS;
     const bool G = TH && i >= Q;
@@ -350,7 +379,7 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
     if constexpr (TH) {  // flow grids have the uniform base state
         ro = A.roff[y];
         to = A.toff[y];
-        if (vy != 0) base = R(vy) * wgt<R>(a <= 4 ? 1 : 5) * __ldg(A.dref + ((G ? 2 : 0) + (vy > 0 ? 0 : 1)) * A.ny + y);
+        if (vy != 0) base = __ldg(A.dref + ((G ? 2 : 0) + (vy > 0 ? 0 : 1)) * A.ny + y);
     }
     dependency_wait(P.early);
 
@@ -365,23 +394,24 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
         for (int s = 0; s < 4; ++s) hy[s] = H[oy[s]];
     }
     const R fc = P.b[own];
-    R v = base;
-    if (vx != 0) v += kx.div(hx);
+    R v = 0;
+    if (vx != 0) v = kx.x(hx, vx);
     if (vy != 0) {
         if constexpr (TH) {
 #pragma unroll
             for (int s = 0; s < 4; ++s) hy[s] = flip(hy[s], G && (gy >> s & 1u) ? ~0u : 0u);
         }
-        v += ky.div(hy);
+        v = ky.y(hy, vy, v);
+        if constexpr (TH) v = add_base(v, R(vy) * wgt<R>(a <= 4 ? 1 : 5), base);
     }
     R d;
     if constexpr (CORR) {
-        d = fc - A.hf * v;
+        d = mad(-A.hf, v, fc);
         if (in) Store<S>::st(static_cast<S*>(G ? A.gout : A.fout) + (unsigned)a * pb + c, d);
         d = Round<S>::of(d);  // the next step starts from the stored value
     } else {
-        if (in) P.b[own] = fc - A.hf * v;
-        d = fc - A.dt * v;
+        if (in) P.b[own] = mad(-A.hf, v, fc);
+        d = mad(-A.dt, v, fc);
     }
     sd[i][lane] = d;
     __syncthreads();
@@ -392,48 +422,63 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
             f[q] = sd[q][lane];
             if constexpr (TH) e[q] = sd[Q + q][lane];
         }
-        CellMom<R, TH> m;
+        typename MomOf<R, TH>::T m;
         m.build(f, e, A, ro, to);
         sm[0][lane] = m.rp;
         sm[1][lane] = m.rho;
         sm[2][lane] = m.ux3;
         sm[3][lane] = m.uy3;
-        sm[4][lane] = m.mx;
-        sm[5][lane] = m.my;
-        sm[6][lane] = A.omh * m.uuneg + A.hF * m.ua3neg;
-        sm[7][lane] = R(3) * A.hF * m.ay;
+        if constexpr (sizeof(R) == 8) {  // formed once, not by every population's thread
+            sm[4][lane] = A.omh * m.uuneg + A.hF * m.ua3neg;
+            sm[5][lane] = A.omgh * m.uuneg;
+            sm[6][lane] = R(3) * A.hF * m.ay;
+        } else {
+            sm[4][lane] = m.uuneg;
+            sm[5][lane] = m.ua3neg;
+            sm[6][lane] = m.ay;
+        }
         if constexpr (TH) {
-            sm[8][lane] = m.Td;
-            sm[9][lane] = m.T;
-            sm[10][lane] = A.omgh * m.uuneg;
+            sm[7][lane] = m.Td;
+            sm[8][lane] = m.T;
         }
     }
     __syncthreads();
-    // h of population a, as CellMom::relax_f / relax_g form it
-    const R w = a == 0 ? wgt<R>(0) : (a <= 4 ? wgt<R>(1) : wgt<R>(5));
-    const R w0 = a == 0 ? wsum<R>(0) : (a <= 4 ? wsum<R>(1) : wsum<R>(5));
-    const R w3 = a <= 4 ? wdir<R>(1) : wdir<R>(5);  // the rest population has no odd part
-    const R k1 = P.k[G], kh = P.kh[G];
-    auto along = [&](int q) {  // c.(sm[q], sm[q + 1])
-        R v = vx == 0 ? R(0) : (vx > 0 ? sm[q][lane] : -sm[q][lane]);
-        if (vy != 0) v += vy > 0 ? sm[q + 1][lane] : -sm[q + 1][lane];
-        return v;
-    };
-    const R cu3 = along(2);
-    R ct = 0;
-    if (!G) {
-        if (vx != 0) ct = vx > 0 ? P.ctx : -P.ctx;
-        if (vy != 0) ct += vy > 0 ? sm[7][lane] : -sm[7][lane];
-    }
-    constexpr int kT = TH ? 8 : 0;  // first thermal moment
-    const R g = cu3 * kh + ct, ev = cu3 * g + sm[G ? kT + 2 : 6][lane];
-    const R wr = w * sm[G ? kT + 1 : 1][lane], dm = w0 * sm[G ? kT : 0][lane] - d;
-    R t;
-    if constexpr (sizeof(R) == 8) t = k1 * dm + wr * (ev + (cu3 * kh + g));
-    else t = k1 * ((G ? wr : w3) * (G ? cu3 : along(4)) + dm) + wr * (ev + ct);
-    if (in) {
-        (CORR ? P.h : P.hs)[own] = d + t;
-        if constexpr (CORR) P.b[own] = d + R(2) * t;
+    if constexpr (sizeof(R) == 8) {
+        // h = d + t of population a, as CellMom forms t
+        const R w = a == 0 ? wgt<R>(0) : (a <= 4 ? wgt<R>(1) : wgt<R>(5));
+        const R k1 = P.k[G], kh = P.kh[G];
+        R cu3 = vx == 0 ? R(0) : (vx > 0 ? sm[2][lane] : -sm[2][lane]);
+        if (vy != 0) cu3 += vy > 0 ? sm[3][lane] : -sm[3][lane];
+        R ct = 0;
+        if (!G) {
+            if (vx != 0) ct = vx > 0 ? P.ctx : -P.ctx;
+            if (vy != 0) ct += vy > 0 ? sm[6][lane] : -sm[6][lane];
+        }
+        constexpr int kT = TH ? 7 : 0;  // first thermal moment
+        const R g = cu3 * kh + ct, ev = cu3 * g + sm[G ? 5 : 4][lane];
+        const R wr = w * sm[G ? kT + 1 : 1][lane], dm = w * sm[G ? kT : 0][lane] - d;
+        const R t = k1 * dm + wr * (ev + (cu3 * kh + g));
+        if (in) {
+            (CORR ? P.h : P.hs)[own] = d + t;
+            if constexpr (CORR) P.b[own] = d + R(2) * t;
+        }
+    } else {
+        pairmath::LaneMom<TH> m;
+        m.rp = sm[0][lane];
+        m.rho = sm[1][lane];
+        m.ux3 = sm[2][lane];
+        m.uy3 = sm[3][lane];
+        m.uuneg = sm[4][lane];
+        m.ua3neg = sm[5][lane];
+        m.ay = sm[6][lane];
+        if constexpr (TH) {
+            m.Td = sm[7][lane];
+            m.T = sm[8][lane];
+        }
+        if (in) {
+            (CORR ? P.h : P.hs)[own] = G ? m.one_g(a, d, A.omgh) : m.one_f(a, d, A, A.omh, A.hF);
+            if constexpr (CORR) P.b[own] = G ? m.one_g(a, d, A.omg) : m.one_f(a, d, A, A.om, A.cf);
+        }
     }
 }
 

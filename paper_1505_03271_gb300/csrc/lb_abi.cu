@@ -129,24 +129,81 @@ bool pair_ok(const lb_grid* G) {
 
 bool has_density_axis(const lb_grid* G) { return G->d.bcx == LB_BC_DENSITY || G->d.bcy == LB_BC_DENSITY; }
 
-// Schedule actually used: AUTO takes a marching kernel (the paired one when
-// it applies) once the grid is wide and tall enough to fill the GPU with
-// strips, else the tile kernel.
-int resolved_kernel(const lb_grid* G) {
-    if (G->fv_kernel != LB_FV_AUTO) return G->fv_kernel;
-    if (G->nx >= 480 && G->ny >= 256 && !G->d.thermal) return pair_ok(G) ? LB_FV_PAIR : LB_FV_MARCH;
-    return pair_ok(G) ? LB_FV_PTILE : LB_FV_TILE;
+// How many waves n CTAs take on `slots` places.
+long long waves(long long n, long long slots) { return (n + slots - 1) / slots; }
+
+// The block march (k_fv_blocks.cu): strip width and rows per CTA, and the
+// time a step takes in microseconds.  A CTA that owns ch rows runs ch / 4 + 4
+// iterations; measured, one takes 1.65 us on a wide flow strip (120 columns,
+// one CTA per SM), 1.8 on two narrow ones (56 columns each, two CTAs per SM;
+// one alone 1.5) and 1.75 on a thermal strip (56 columns).
+struct March {
+    bool wide;
+    int chunk;
+    double us;
+};
+March march_plan(const lb_grid* G, int chunk) {
+    March best{true, 0, 1e300};
+    const bool th = G->d.thermal != 0;
+    for (int wide = th ? 1 : 0; wide < 2; ++wide) {
+        const int width = blocks_width(th, wide != 0);
+        const long long strips = (G->nx + width - 1) / width;
+        auto cost = [&](long long ch) {
+            const long long n = strips * ((G->ny + ch - 1) / ch);
+            const double it = th ? 1.75 : wide ? 1.65 : n <= G->sms ? 1.5 : 1.8;
+            return waves(n, (long long)G->sms * (wide ? 1 : 2)) * (ch / 4 + 4) * it + 1.5;
+        };
+        auto take = [&](long long ch) {
+            ch = (ch + 3) / 4 * 4;
+            const double us = cost(ch);
+            if (us < best.us) best = {wide != 0, (int)ch, us};
+        };
+        if (chunk > 0) take(chunk);
+        else
+            for (long long w = 1; w <= 8; ++w) {  // the tallest chunks that fill w waves
+                const long long chunks = w * G->sms * (wide ? 1 : 2) / strips;
+                take(chunks < 1 ? G->ny : (G->ny + chunks - 1) / chunks);
+            }
+    }
+    return best;
 }
 
-// Rows per CTA of the marching kernels: one wave of resident CTAs.
+// The paired tile (lb_block.cuh): shape and time.  A wave of tiles takes 6.5
+// us at 16 rows and 6.2 at 14 (flow, two CTAs per SM), 6.7 and 6.55 on
+// thermal grids (one per SM); 16 x 16 thermal tiles 5.7 in a single wave.
+struct Tile {
+    int shape;
+    double us;
+};
+Tile tile_plan(const lb_grid* G) {
+    const bool th = G->d.thermal != 0;
+    const long long cols = (G->nx + 31) / 32, slots = (long long)G->sms * (th ? 1 : 2);
+    Tile t{th ? 512 : 0, waves(cols * ((G->ny + 15) / 16), slots) * (th ? 6.7 : 6.5) + 1.5};
+    const double us14 = waves(cols * ((G->ny + 13) / 14), slots) * (th ? 6.55 : 6.2) + 1.5;
+    if (us14 < t.us) t = {th ? 526 : 14, us14};
+    if (th && (long long)((G->nx + 15) / 16) * ((G->ny + 15) / 16) <= G->sms && t.us > 7.2) t = {16, 7.2};
+    return t;
+}
+
+// Schedule actually used: AUTO takes the paired tile or the block march,
+// whichever those figures put first (1024 x 1024 FP32: tile 45.7 us, march
+// 35.7; 512 x 512: 14.3 and 16.5; thermal 16-bit 1024 x 1024: 92 and 65), and
+// on grids they do not serve the scalar march once its strips fill the GPU,
+// else the scalar tile.
+int resolved_kernel(const lb_grid* G) {
+    if (G->fv_kernel != LB_FV_AUTO) return G->fv_kernel;
+    if (pair_ok(G)) return march_plan(G, 0).us < tile_plan(G).us ? LB_FV_PAIR : LB_FV_PTILE;
+    return G->nx >= 480 && G->ny >= 256 && !G->d.thermal ? LB_FV_MARCH : LB_FV_TILE;
+}
+
+// Rows per CTA of the marching kernels.
 int resolved_chunk(const lb_grid* G) {
+    if (resolved_kernel(G) == LB_FV_PAIR) return march_plan(G, G->fv_chunk).chunk;
     if (G->fv_chunk > 0) return G->fv_chunk;
     const bool th = G->d.thermal != 0;
-    const bool pr = resolved_kernel(G) == LB_FV_PAIR;
-    const int width = pr ? pair_width() : march_width(G->prec, th);
+    const int width = march_width(G->prec, th);
     const int strips = (G->nx + width - 1) / width;
-    const size_t smem = pr ? pair_smem(th) : march_smem(G->prec, th);
-    int per_sm = (int)(227 * 1024 / smem);
+    int per_sm = (int)(227 * 1024 / march_smem(G->prec, th));
     if (per_sm < 1) per_sm = 1;
     if (per_sm > 4) per_sm = 4;
     // about four waves of resident CTAs: short marches balance better than
@@ -157,6 +214,8 @@ int resolved_chunk(const lb_grid* G) {
     int ch = (int)((G->ny + chunks - 1) / chunks);
     return ch < 32 ? 32 : ch;
 }
+
+int resolved_shape(const lb_grid* G) { return G->fv_kernel == LB_FV_PTILE ? G->fv_chunk : tile_plan(G).shape; }
 
 // The split schedule's two FP32 buffers (NQ planes each), allocated on
 // first use.
@@ -186,16 +245,18 @@ cudaError_t launch_fv_step(lb_grid* G) {
         A.xfc = G->xfc;
         return launch_fv_split(G->prec, th, &A, G->fv_chunk, G->stream);
     }
-    if (k == LB_FV_PAIR) return launch_fv_pair(G->prec, th, &A, resolved_chunk(G), G->stream);
-    if (k == LB_FV_PTILE) return launch_fv_ptile(G->prec, th, &A, G->fv_kernel == LB_FV_PTILE ? G->fv_chunk : 0,
-                                                 G->stream);
+    if (k == LB_FV_PAIR) {
+        const March m = march_plan(G, G->fv_kernel == LB_FV_PAIR ? G->fv_chunk : 0);
+        return launch_fv_blocks(G->prec, th, &A, m.chunk, m.wide, G->stream);
+    }
+    if (k == LB_FV_PTILE) return launch_fv_ptile(G->prec, th, &A, resolved_shape(G), G->stream);
     if (k == LB_FV_MARCH) return launch_fv_march(G->prec, th, &A, resolved_chunk(G), G->stream);
     return launch_fv(G->prec, th, &A, G->fv_kernel == LB_FV_TILE ? G->fv_chunk : 0, G->stream);
 }
 
 // Whether lb_step_fv runs the two-launch step of k_fv_phase.cu: FP64 grids
 // of every size (the fused kernels recompute on the scarce FP64 pipe), and
-// FP32-math grids up to 128 cells per SM (thermal: 64), where the fused tile
+// x-periodic FP32-math grids up to 128 cells per SM (thermal: 64), where the fused tile
 // leaves most SMs idle: 128 x 128 FP32 takes 4.4 us a step against 6.1,
 // 192 x 192 8.1 against 6.3; thermal 96 x 96 4.9 against 9.1, 128 x 128 8.9
 // against 9.1.  Its kernels address a pair of planes with 32-bit offsets.
@@ -204,7 +265,7 @@ bool phase_applies(const lb_grid* G) {
     const bool f64 = G->prec == Prec::F64;
     if (3ULL * G->plane * (f64 ? 8 : 4) >= 1ULL << 32) return false;
     if (G->fv_kernel != LB_FV_AUTO) return G->fv_kernel == LB_FV_TILE && G->fv_chunk == 2;
-    return f64 || (G->d.thermal ? 2LL : 1LL) * G->nx * G->ny <= 128LL * G->sms;
+    return f64 || (pair_ok(G) && (G->d.thermal ? 2LL : 1LL) * G->nx * G->ny <= 128LL * G->sms);
 }
 
 // The two-launch step's fields, allocated on first use; false where that is
@@ -718,8 +779,9 @@ lb_status lb_get_fv_schedule(lb_grid* G, int* kernel, int* chunk) {
     if (kernel) *kernel = resolved_kernel(G);
     if (chunk) {
         const int k = resolved_kernel(G);
-        *chunk = (k == LB_FV_TILE || k == LB_FV_PTILE || k == LB_FV_SPLIT) ? (G->fv_kernel == k ? G->fv_chunk : 0)
-                                                                            : resolved_chunk(G);
+        *chunk = k == LB_FV_PTILE                        ? resolved_shape(G)
+                 : k == LB_FV_TILE || k == LB_FV_SPLIT ? (G->fv_kernel == k ? G->fv_chunk : 0)
+                                                       : resolved_chunk(G);
     }
     return LB_OK;
 }

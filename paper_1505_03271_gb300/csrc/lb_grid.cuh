@@ -71,7 +71,7 @@ struct Axis {
     // Per cell, for c > 0 and then for c < 0, the two-launch step's weights
     // of c (Phi_e - Phi_w) / dx.  FP64: K[4] with the sum K_s h_s over the
     // nodes (from -2 for c > 0, from -1 for c < 0).  FP32: the west and the
-    // east face's three weights, c / dx and a pad.
+    // east face's three weights, 1 / dx and a pad.
     std::vector<double> cell_weights(bool f32) const {
         const int m = f32 ? 8 : 4;
         std::vector<double> t(2 * (size_t)m * n, 0.0);
@@ -84,7 +84,7 @@ struct Axis {
                 double* k = &t[(size_t)m * (2 * i + sg)];
                 if (f32) {
                     for (int r = 0; r < 3; ++r) k[r] = w[r], k[3 + r] = e[r];
-                    k[6] = s;
+                    k[6] = 1.0 / d[i];
                 } else {
                     k[0] = -w[0] * s;
                     k[1] = (e[0] - w[1]) * s;

@@ -206,10 +206,11 @@ void tile_shape(Prec p, bool thermal, int* tx, int* ty);
 cudaError_t launch_fv_march(Prec p, bool thermal, const void* args, int chunk, cudaStream_t s);
 int march_width(Prec p, bool thermal);
 size_t march_smem(Prec p, bool thermal);
-// paired-column marching FV kernel (FP32 arithmetic, x-periodic grids only)
-cudaError_t launch_fv_pair(Prec p, bool thermal, const void* args, int chunk, cudaStream_t s);
-int pair_width();
-size_t pair_smem(bool thermal);
+// march in blocks of four rows, packed FP32 pairs (x-periodic grids only): strips of
+// blocks_width() columns, `chunk` rows per CTA (rounded up to a multiple of 4);
+// wide: one CTA per SM, else (flow grids) two of half the strip
+cudaError_t launch_fv_blocks(Prec p, bool thermal, const void* args, int chunk, bool wide, cudaStream_t s);
+int blocks_width(bool thermal, bool wide);
 // paired tile kernel: shape 0 = 32 x 16, 16 = 16 x 16 (x-periodic, FP32 arithmetic)
 cudaError_t launch_fv_ptile(Prec p, bool thermal, const void* args, int shape, cudaStream_t s);
 // split paired schedule: two launches per step (collision + predictor, corrector),

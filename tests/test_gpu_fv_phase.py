@@ -2,7 +2,8 @@
 grids) element by element against the FP64 oracle, on both of its forms and
 at the sizes where they change: one population per thread at 8 and at 32
 cells per CTA, one cell per thread on larger FP64 grids; periodic and wall
-axes, ragged last CTAs, axes shorter than the stencil."""
+axes, ragged last CTAs, axes shorter than the stencil.  And the packed FP32
+schedules (tile, block march, two launches) against each other, bit for bit."""
 import numpy as np
 import pytest
 
@@ -56,22 +57,31 @@ def test_two_launch_step(lbgpu, oracle, case, store):
             assert np.abs(a - b).max() <= tol
 
 
-@pytest.mark.parametrize("store", ["f16dev", "bf16dev"])
-def test_two_launch_step_16bit(lbgpu, store):
-    """16-bit storage: the two launches and the paired tile round the same
-    states, so after one step they differ by at most one rounding of the
-    stored deviations (2^-10 and 2^-7 of the largest)."""
-    out = []
-    for sched in ((4, 0), (1, 2)):
-        g = lbgpu.Grid(40, 36, sy=1, stretch_y=2.0, bcy=1, thermal=True, store=store)
-        g.init(tau=0.1, tau_g=0.1, dt=0.05, beta=1e-3, grav=1.0, T0=1.0, T_bot=1.5, T_top=0.5, kind=lbgpu.LB_INIT_RB,
-               amp=1e-2, seed=5)
-        g.set_pops(inputs.random_populations(40, 36, seed=2, amp=0.1), inputs.random_populations(40, 36, seed=3, amp=0.1))
-        out.append(g.set_fv_schedule(*sched).step_fv(1).get_pops())
-    ulp = 2.0 ** -10 if store == "f16dev" else 2.0 ** -7
-    w = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
-    for a, b in zip(*out):
-        assert np.abs(a - b).max() <= ulp * max(np.abs(a - w).max(), 0.05)
+PAIRED = [  # x-periodic grids: ragged tiles and blocks, walls in every position of a block, axes shorter than a stencil
+    dict(nx=70, ny=37), dict(nx=45, ny=33, sy=1, stretch_y=2.0, bcy=1), dict(nx=5, ny=3), dict(nx=64, ny=2, bcy=1),
+    dict(nx=1, ny=9), dict(nx=33, ny=4, bcy=1), dict(nx=40, ny=5, sy=1, stretch_y=2.0, bcy=1), dict(nx=61, ny=6, bcy=1),
+    dict(nx=50, ny=7, sy=1, stretch_y=2.0, bcy=1), dict(nx=250, ny=66, sy=1, stretch_y=2.0, bcy=1)]
+
+
+@pytest.mark.parametrize("store", ["f32", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("thermal", [False, True], ids=["flow", "thermal"])
+@pytest.mark.parametrize("case", PAIRED, ids=lambda c: "-".join(f"{k}{v}" for k, v in c.items()))
+def test_packed_schedules_are_one_step(lbgpu, case, thermal, store):
+    """The paired tile, the block march (chunks of one block, of several, of
+    the whole grid, the automatic one) and the two-launch step form the same
+    values in the same order: equal populations, bit for bit."""
+    kw = dict(tau=0.3, dt=0.05, ax=2e-4, ay=-1e-4)
+    if thermal:
+        kw.update(tau_g=0.25, beta=1e-2, grav=1.0, T0=1.0, T_bot=1.3, T_top=0.8)
+    nx, ny, out = case["nx"], case["ny"], []
+    grid = lbgpu.Grid(**case, thermal=thermal, store=store).init(**kw)
+    f = inputs.random_populations(nx, ny, seed=1, amp=0.2)
+    g = inputs.random_populations(nx, ny, seed=2, amp=0.2) if thermal else None
+    for sched in ((4, 0), (4, 526), (4, 16), (3, 4), (3, 8), (3, 12), (3, 64), (3, 0), (1, 2)):
+        out.append(grid.set_pops(f, g).set_fv_schedule(*sched).step_fv(3).get_pops())
+    for o in out[1:]:
+        assert np.array_equal(o[0], out[0][0])
+        assert not thermal or np.array_equal(o[1], out[0][1])
 
 
 @pytest.mark.parametrize("nx,ny,thermal,store,two", [

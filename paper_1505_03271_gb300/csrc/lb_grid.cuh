@@ -138,6 +138,7 @@ struct lb_grid {
     long long plane = 0;
     lbgb::Axis ax, ay;
     double dmin = 0;
+    void* arena = nullptr;  // the one allocation the pointers below lead into, unless they say otherwise
     void* f[2] = {nullptr, nullptr};
     void* g[2] = {nullptr, nullptr};
     int cur = 0;
@@ -226,5 +227,8 @@ inline StepArgs<R> step_args(const lb_grid* G, double dt) {
     A.xfc = G->xfc;
     return A;
 }
+
+// the closing figures of a served request (lb_abi.cu)
+lb_status final_figures(lb_grid* G, double* mass, double* nu_vol, double* nu_bot, double* nu_top);
 
 }  // namespace lbgb

@@ -186,11 +186,7 @@ void retire(lb_server* S, Active& a, lb_status status) {
     r.cells = (long long)a.req.grid.nx * a.req.grid.ny;
     r.status = status;
     if (status == LB_OK) {
-        double mass = 0;
-        lb_status s = lb_conservation(a.grid, &mass, nullptr, nullptr, nullptr);
-        r.mass = mass;
-        if (s == LB_OK && S->thermal) s = lb_nusselt(a.grid, &r.nu_vol, &r.nu_bot, &r.nu_top);
-        r.status = s;
+        r.status = final_figures(a.grid, &r.mass, &r.nu_vol, &r.nu_bot, &r.nu_top);
     }
     r.t_done = S->now();
     lb_destroy(a.grid);

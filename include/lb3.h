@@ -78,7 +78,8 @@ lb_status lb3_init(lb3_grid* grid, const lb3_params* params, const lb3_init_desc
 /* nsteps FV steps, Eq. (semi-heun): four kernel launches per step (the
  * collision pass with h and its z ghost planes, the predictor's flux pass,
  * the moments of f~* with h* and its ghost planes, the corrector's flux
- * pass). */
+ * pass), or two where LB3_FV_AUTO allows them (the predictor's flux pass
+ * goes on to h*, the corrector's to the next h). */
 lb_status lb3_step_fv(lb3_grid* grid, int nsteps);
 
 /* Flux passes of lb3_step_fv (the QUICK divergence of Sec. II B 3):
@@ -90,6 +91,9 @@ lb_status lb3_step_fv(lb3_grid* grid, int nsteps);
  *                  rows are a multiple of 16 bytes (nx >= 4 for FP32, >= 2
  *                  for FP64);
  *   LB3_FV_AUTO:   STAGED where the grid allows it, else PLAIN (default).
+ *                On small FP32 grids with the default staged shape its
+ *                steps run as two passes that give STAGED's state bit for
+ *                bit.
  * Both give the same step up to the rounding of the folded face weights.
  * lb3_set_fv_schedule returns LB_ERR_ARG for STAGED on a grid it does not
  * serve; lb3_get_fv_schedule writes the passes a step runs (PLAIN or

@@ -372,6 +372,180 @@ __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 1 : 2) k3_star(const Arg
     zghosts<R, TH>(A.HS, A.HGS, i, j, k, A);
 }
 
+// ---- FV in two passes (FP32; the grids the staged flux passes serve) ----
+// A thread carries one cell through both sides of a flux pass, all of its
+// populations at once:
+//   k3_predict  A[h^n] -> f~* -> its moments -> h*; f~ + Coll - dt/2 A[h^n]
+//   k3_correct  A[h*] -> f~^(n+1) -> its moments -> h^(n+1), f~ + Coll
+// so f~* never goes through memory, and the state only on a call's last step
+// (LAST), which needs nothing else: 304 values per cell and step instead of
+// the 456 of four passes.  k3_pre forms h and f~ + Coll before the first step.
+// Stencil nodes come through L1 (x, y within the block) and L2: a block of
+// 32 x BY x BZ cells, whose 8 loads per population are independent over 38
+// populations.  Every value is formed with the operations, and in the order,
+// of the four passes (folded weights as in k3_staged.cu), so the state is the
+// same bit for bit.
+// Up to 150000 thermal cells the state stays in L2 and half the launches
+// count (lb3_abi.cu has the times); on 128 x 128 x 64 the nodes' latency at 16
+// warps per SM holds both passes to 3.5 TB/s of HBM, and four passes are
+// faster.  k3_predict loads its f~ + Coll ahead of the first store: 597 -> 377
+// us a step there.
+__device__ __forceinline__ void fold_axis(const AxisMetric<float>& M, int m, int cv, float* K) {
+    const int q0 = cv > 0 ? 0 : 3;
+    float w[3], e[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        w[r] = M.row(q0 + r, m);
+        e[r] = M.row(q0 + r, m + 1);
+    }
+    const float s = float(cv) * M.invd(m);
+    K[0] = -w[0] * s;
+    K[1] = (e[0] - w[1]) * s;
+    K[2] = (e[1] - w[2]) * s;
+    K[3] = e[2] * s;
+}
+
+// A cell's stencil: element offsets of nodes -2..2 per axis in a padded
+// population, and the folded weights for c > 0 and c < 0.
+struct Cross {
+    unsigned o[3][5];
+    float kp[3][4], km[3][4];
+    __device__ __forceinline__ void set(const Args3<float>& A, int i, int j, int k) {
+        const unsigned own = (unsigned)padded3(A.n, i, j, k);
+        const unsigned st[3] = {1u, (unsigned)A.n[0], (unsigned)A.n[0] * A.n[1]};
+        const int pos[3] = {i, j, k};
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+#pragma unroll
+            for (int s = -2; s <= 2; ++s) {
+                int q = pos[ax] + s;
+                if (ax < 2 && (q < 0 || q >= A.n[ax])) q = ((q % A.n[ax]) + A.n[ax]) % A.n[ax];  // z has ghost planes
+                o[ax][s + 2] = own + (unsigned)(q - pos[ax]) * st[ax];
+            }
+            fold_axis(A.m[ax], pos[ax], 1, kp[ax]);
+            fold_axis(A.m[ax], pos[ax], -1, km[ax]);
+        }
+    }
+    template <int a>
+    __device__ __forceinline__ float flux(const float* P) const {
+        constexpr int c[3] = {c3x(a), c3y(a), c3z(a)};
+        float v = 0.0f;
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            if (c[ax] == 0) continue;
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                v = __fmaf_rn(c[ax] > 0 ? kp[ax][s] : km[ax][s], __ldg(P + o[ax][s + (c[ax] > 0 ? 0 : 1)]), v);
+        }
+        return v;
+    }
+};
+
+template <bool TH, int a = 0, typename F>
+__device__ __forceinline__ void each_flux(const Cross& X, const float* H, const float* HG, long long NP, F&& use) {
+    use(a, false, X.flux<a>(H + a * NP));
+    if constexpr (TH) use(a, true, X.flux<a>(HG + a * NP));
+    if constexpr (a + 1 < Q3) each_flux<TH, a + 1>(X, H, HG, NP, use);
+}
+
+template <bool TH, int BY, int BZ>
+__device__ __forceinline__ bool block_cell(const int* n, int& i, int& j, int& k) {
+    i = blockIdx.x * 32 + threadIdx.x;
+    j = blockIdx.y * BY + threadIdx.y;
+    k = blockIdx.z * BZ + threadIdx.z;
+    return i < n[0] && j < n[1] && k < n[2];
+}
+
+// zghosts of a block whose threads are on several planes
+template <bool TH>
+__device__ __forceinline__ void zghost_cell(float* P, float* PG, int i, int j, int k, const Args3<float>& A) {
+    if (k >= 2 && k < A.n[2] - 2) return;
+    const long long cp = padded3(A.n, i, j, k);
+    for (int a = 0; a < Q3; ++a) {
+        zghost(P, a, P[a * A.NP + cp], i, j, k, false, A);
+        if constexpr (TH) zghost(PG, a, PG[a * A.NP + cp], i, j, k, true, A);
+    }
+}
+
+template <bool TH, int BY, int BZ>
+__global__ void __launch_bounds__(32 * BY * BZ, 512 / (32 * BY * BZ)) k3_predict(const Args3<float> A) {
+    int i, j, k;
+    if (!block_cell<TH, BY, BZ>(A.n, i, j, k)) return;
+    Cross X;
+    X.set(A, i, j, k);
+    const long long c = cell3(A.n, i, j, k), N = A.N, cp = padded3(A.n, i, j, k), NP = A.NP;
+    // f~ + Coll first, all of it: behind the stores below each of these loads
+    // would wait alone
+    float fs[Q3], es[Q3];
+#pragma unroll
+    for (int a = 0; a < Q3; ++a) {
+        fs[a] = A.FC[a * N + c];
+        if constexpr (TH) es[a] = A.GC[a * N + c];
+    }
+    each_flux<TH>(X, A.H, A.HG, NP, [&](int a, bool g, float v) {
+        float& f = (g ? es : fs)[a];
+        (g ? A.GC : A.FC)[a * N + c] = __fmaf_rn(-A.hf, v, f);
+        f = __fmaf_rn(-A.dt, v, f);
+    });
+    float r = 0, jx = 0, jy = 0, jz = 0, td = 0;
+#pragma unroll
+    for (int a = 0; a < Q3; ++a) {
+        r += fs[a];
+        jx += float(c3x(a)) * fs[a];
+        jy += float(c3y(a)) * fs[a];
+        jz += float(c3z(a)) * fs[a];
+        if constexpr (TH) td += es[a];
+    }
+    Cell3<float, TH> m;
+    m.from_sums(r, jx, jy, jz, td, A);
+#pragma unroll
+    for (int a = 0; a < Q3; ++a) {
+        float feqd, F, geqd;
+        m.eq(a, A, feqd, F, geqd);
+        A.HS[a * NP + cp] = fs[a] + A.omh * (feqd - fs[a]) + A.hF * F;
+        if constexpr (TH) A.HGS[a * NP + cp] = es[a] + A.omgh * (geqd - es[a]);
+    }
+    zghost_cell<TH>(A.HS, A.HGS, i, j, k, A);
+}
+
+template <bool TH, bool LAST, int BY, int BZ>
+__global__ void __launch_bounds__(32 * BY * BZ, 512 / (32 * BY * BZ)) k3_correct(const Args3<float> A) {
+    int i, j, k;
+    if (!block_cell<TH, BY, BZ>(A.n, i, j, k)) return;
+    Cross X;
+    X.set(A, i, j, k);
+    const long long c = cell3(A.n, i, j, k), N = A.N, cp = padded3(A.n, i, j, k), NP = A.NP;
+    float d[Q3], e[Q3];
+#pragma unroll
+    for (int a = 0; a < Q3; ++a) {
+        d[a] = A.FC[a * N + c];
+        if constexpr (TH) e[a] = A.GC[a * N + c];
+    }
+    each_flux<TH>(X, A.HS, A.HGS, NP, [&](int a, bool g, float v) {
+        float& f = (g ? e : d)[a];
+        f = __fmaf_rn(-A.hf, v, f);
+        if constexpr (LAST) static_cast<float*>(g ? A.gout : A.fout)[a * N + c] = f;
+    });
+    if constexpr (!LAST) {
+        Cell3<float, TH> m;
+        m.moments(d, e, A);
+#pragma unroll
+        for (int a = 0; a < Q3; ++a) {
+            float feqd, F, geqd;
+            m.eq(a, A, feqd, F, geqd);
+            const float neq = feqd - d[a];
+            A.H[a * NP + cp] = d[a] + A.omh * neq + A.hF * F;
+            A.FC[a * N + c] = d[a] + A.om * neq + A.cf * F;
+            if constexpr (TH) {
+                const float neqg = geqd - e[a];
+                A.HG[a * NP + cp] = e[a] + A.omgh * neqg;
+                A.GC[a * N + c] = e[a] + A.omg * neqg;
+            }
+        }
+        zghost_cell<TH>(A.H, A.HG, i, j, k, A);
+    }
+}
+
 // ---- ST: collide and push, Eq. (ST) at dt = dx = 1 ----
 template <typename R, typename S, bool TH>
 __global__ void __launch_bounds__(256) k3_st(const Args3<R> A) {
@@ -542,6 +716,24 @@ cudaError_t run_fv3(const Args3<R>& A, bool staged, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// nsteps steps in two passes each; the state after the last goes to fout, gout
+template <bool TH>
+cudaError_t run_fv3_passes(const Args3<float>& A, int nsteps, cudaStream_t s) {
+    constexpr int BY = 2, BZ = 1;
+    k3_pre<float, float, TH><<<grid3(A.n), dim3(32, 8), 0, s>>>(A);
+    count_launch();
+    const dim3 b(32, BY, BZ), g((A.n[0] + 31) / 32, (A.n[1] + BY - 1) / BY, (A.n[2] + BZ - 1) / BZ);
+    for (int q = 0; q < nsteps; ++q) {
+        k3_predict<TH, BY, BZ><<<g, b, 0, s>>>(A);
+        if (q + 1 < nsteps) k3_correct<TH, false, BY, BZ><<<g, b, 0, s>>>(A);
+        else k3_correct<TH, true, BY, BZ><<<g, b, 0, s>>>(A);
+        for (int l = 0; l < 2; ++l) count_launch();
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 template <typename R, typename S, bool TH>
 cudaError_t run_st3(const Args3<R>& A, cudaStream_t s) {
     k3_st<R, S, TH><<<grid3(A.n), dim3(32, 8), 0, s>>>(A);
@@ -561,6 +753,11 @@ cudaError_t launch3_fv(Prec p, bool th, bool staged, const void* args, cudaStrea
         return th ? run_fv3<float, float, true>(A, staged, s) : run_fv3<float, float, false>(A, staged, s);
     }
     return cudaErrorInvalidValue;
+}
+
+cudaError_t launch3_fv_passes(bool th, const void* args, int nsteps, cudaStream_t s) {
+    const auto& A = *static_cast<const Args3<float>*>(args);
+    return th ? run_fv3_passes<true>(A, nsteps, s) : run_fv3_passes<false>(A, nsteps, s);
 }
 
 cudaError_t launch3_st(Prec p, bool th, const void* args, cudaStream_t s) {

@@ -91,6 +91,8 @@ struct Aux3 {
 // One FV step.  staged: run the flux passes of k3_staged.cu (the grid must
 // pass adv3_staged_ok).
 cudaError_t launch3_fv(Prec p, bool th, bool staged, const void* args, cudaStream_t s);
+// nsteps FP32 FV steps in two passes each (k3.cu); the grid must pass adv3_staged_ok.
+cudaError_t launch3_fv_passes(bool th, const void* args, int nsteps, cudaStream_t s);
 // The staged flux pass (k3_staged.cu): whether it serves a grid, and one launch
 // (corr: the corrector's pass; np: 19 or 38 populations).
 bool adv3_staged_ok(const int* n, const int* bc, Prec p);

@@ -95,6 +95,18 @@ bool staged3(const lb3_grid* G) {
     return G->fv_sched == LB3_FV_STAGED || (G->fv_sched == LB3_FV_AUTO && staged_ok3(G));
 }
 
+// whether AUTO's staged steps run as the two passes of k3.cu, whose values are
+// theirs bit for bit: FP32, no staged shape asked for and not under the test
+// hook of the staged passes' waits, up to 150000 thermal or 300000 flow cells, where
+// four launches of few CTAs leave the GPU waiting (thermal 32 x 40 x 20: 27 us
+// a step against 43, 64 x 64 x 32 50 against 59, 128 x 48 x 24 64 against 72,
+// flow 64 x 64 x 64 42 against 56;
+// thermal 128 x 128 x 64, where the passes stream from HBM, 362 against 335)
+bool passes3(const lb3_grid* G) {
+    return G->fv_sched == LB3_FV_AUTO && G->prec == Prec::F32 && staged_ok3(G) && !G->drop_copy && !G->sshape[0] &&
+           !G->sshape[1] && !G->sshape[2] && (G->d.thermal ? 2 : 1) * G->N <= 300000;
+}
+
 // LB_ERR_TIMEOUT (and the grid poisoned) when a staged pass reported a wait
 // that ran out; synchronises the grid's stream.
 lb_status wait_status3(lb3_grid* G) {
@@ -354,6 +366,12 @@ lb_status lb3_step_fv(lb3_grid* G, int nsteps) {
     if (s != LB_OK) return s;
     if (nsteps < 0) return fail3(LB_ERR_ARG, "nsteps must be >= 0");
     Dev3 dg(G->device);
+    if (passes3(G) && nsteps > 0) {
+        Args3<float> A = args3<float>(G, false);
+        CK3(launch3_fv_passes(G->d.thermal != 0, &A, nsteps, G->stream));
+        G->cur ^= 1;  // only the last step writes the state
+        return LB_OK;
+    }
     for (int k = 0; k < nsteps; ++k) CK3(fv3_step(G));
     return LB_OK;
 }

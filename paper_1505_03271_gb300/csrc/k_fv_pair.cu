@@ -346,10 +346,13 @@ cudaError_t launch_fv_split(Prec p, bool th, const void* args, int shape, cudaSt
 template <typename S, bool TH, int TX, int TY, int NTH>
 __global__ void __launch_bounds__(NTH)
 k_fv_ptile_batched(const BatchReq<float>* reqs, const int4* tiles, const int* ntiles, const int k) {
-    if ((int)blockIdx.x >= *ntiles) return;
-    const int4 t = tiles[blockIdx.x];
+    const bool listed = (int)blockIdx.x < *ntiles;
+    const int4 t = tiles[listed ? blockIdx.x : 0];
     const BatchReq<float>& B = reqs[t.x];
-    if (k >= B.remaining) return;
+    if (!listed || k >= B.remaining) {
+        chain_wait();
+        return;
+    }
     StepArgs<float> A = B.args;
     const int p = (B.parity + k) & 1;
     A.fin = B.f[p];
@@ -370,10 +373,10 @@ static cudaError_t run_ptile_batched(const void* reqs, const int4* tiles, const 
         cudaError_t e = set_max_smem((const void*)k_fv_ptile_batched<S, TH, 32, 16, NTH>, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_fv_ptile_batched<S, TH, 32, 16, NTH><<<capacity, NTH, smem, s>>>(static_cast<const BatchReq<float>*>(reqs),
-                                                                      tiles, ntiles, k);
+    const cudaError_t e = launch_chained(k_fv_ptile_batched<S, TH, 32, 16, NTH>, dim3(capacity), NTH, smem, s,
+                                         static_cast<const BatchReq<float>*>(reqs), tiles, ntiles, k);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_fv_ptile_batched(Prec p, bool th, const void* reqs, const int4* tiles, const int* ntiles,
@@ -402,9 +405,9 @@ static cudaError_t run_ptile(const void* vargs, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     dim3 grid((A.nx + TX - 1) / TX, (A.ny + TY - 1) / TY);
-    k_fv_ptile<S, TH, TX, TY, NTH, MINB, RC><<<grid, NTH, smem, s>>>(A);
+    const cudaError_t e = launch_chained(k_fv_ptile<S, TH, TX, TY, NTH, MINB, RC>, grid, NTH, smem, s, A);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 // shape: 0 = 32 x 16 tiles, 256 threads; 14 = 32 x 14, 256 threads;

@@ -13,8 +13,8 @@
 //     cells instead of 5 R, and a face between two of its rows is formed once;
 //   - the wall's ghost rows are written by the threads that hold the rows they
 //     mirror, so a step has two barriers, not four.
-// Step times before and after: channel 256 x 512 FP32 9.0 -> 8.1 us (32 x 14),
-// 512 x 512 16.3 -> 14.3; thermal 16-bit 256 x 256 9.2 -> 7.8 (32 x 14, 512
+// Step times before and after: channel 256 x 512 FP32 9.0 -> 7.7 us (32 x 14),
+// 512 x 512 16.3 -> 13.9; thermal 16-bit 256 x 256 9.2 -> 7.6 (32 x 14, 512
 // threads), 512 x 512 32 -> 27 (where the march of k_fv_blocks.cu takes 23).
 #pragma once
 
@@ -232,6 +232,8 @@ __device__ __forceinline__ void tile_step(const StepArgs<float>& A, const int x0
             sCol[(e - BH) * 5 + part] = __ldg(reinterpret_cast<const float4*>(A.coltab) + 5 * gxl + part);
         }
     }
+
+    chain_wait();
 
     // ---- A: time level n on tile + 4, two columns per thread ----
     constexpr int EP = (TX + 8) / 2;

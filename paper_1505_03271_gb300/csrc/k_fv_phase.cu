@@ -20,9 +20,9 @@
 // 8 of 152 SMs, is bound by the FP64 pipe of those few SMs.  Here nothing is
 // evaluated twice, a warp is 32 cells (or 32 populations of a few cells), and
 // each axis' QUICK divergence is four multiply-adds with folded weights.
-// FP64 step, fused tile -> this: 1 x 64 132 -> 7.4 us, 64 x 64 132 -> 8.7 us,
-// 1024 x 1024 2011 -> 649 us (0.52 -> 1.62 GLUPS).  FP32: 64 x 64 6.1 -> 3.4
-// us, thermal 64 x 64 (16-bit) 9.0 -> 4.0 us.
+// FP64 step, fused tile -> this: 1 x 64 132 -> 7.3 us, 64 x 64 132 -> 8.7 us,
+// 1024 x 1024 2011 -> 654 us (0.52 -> 1.60 GLUPS).  FP32: 64 x 64 6.1 -> 3.7
+// us, thermal 64 x 64 (16-bit) 9.0 -> 4.3 us.
 #include "lb_pair.cuh"
 #include "lb_phase.cuh"
 
@@ -195,7 +195,7 @@ __device__ __forceinline__ void store_h(const R* d, const R* e, const PhaseArgs<
 // be resident, their indices and weights loaded, before the previous kernel
 // has finished; every kernel waits here for its completion before it touches
 // a field.  early lets the next kernel in at once, which hides its start-up
-// where both fit (64 x 64, FP32: 3.4 us a step, 4.4 without); on grids that
+// where both fit (64 x 64, FP32: 1.0 us of a 4.4 us step); on grids that
 // fill the SMs its waiting CTAs would unbalance the running kernel's
 // (256 x 256, FP64: 72 us against 48), which then releases it as it ends.
 __device__ __forceinline__ void dependency_wait(int early) {
@@ -485,16 +485,7 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
 template <typename K, typename R>
 cudaError_t launch_pdl(K kernel, const PhaseArgs<R>& P, int block, int cells, cudaStream_t s) {
     const long long n = (long long)P.s.nx * P.s.ny;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)((n + cells - 1) / cells));
-    cfg.blockDim = dim3(block);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P);
+    const cudaError_t e = launch_chained(kernel, dim3((unsigned)((n + cells - 1) / cells)), block, 0, s, P);
     count_launch();
     return e;
 }

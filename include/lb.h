@@ -300,7 +300,9 @@ lb_status lb_conservation_noalloc(const float* f, const float* g, int nx, int ny
  * memory), advances all active requests together by up to
  * steps_per_launch FV steps (Eq. (semi-heun)) in one batched kernel per
  * step over a device table of (request, tile) entries, replayed from a
- * captured CUDA graph, and retires the requests that are done.  Every tile
+ * captured CUDA graph, and retires the requests that are done.  Requests
+ * large enough to fill the GPU (thermal from about 512 x 512) step in
+ * launches of their own on LB_FV_PAIR, which gives the same bits.  Every tile
  * is stepped by the same code whatever else is in the table, so a request's
  * result is bit-for-bit the same alone and in any batch; it is the
  * LB_FV_TILE step of lb_step_fv (equal up to FP32 rounding, since the two are

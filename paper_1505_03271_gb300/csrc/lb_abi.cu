@@ -185,8 +185,9 @@ Tile tile_plan(const lb_grid* G) {
 }
 
 // Schedule actually used: AUTO takes the paired tile or the block march,
-// whichever those figures put first (1024 x 1024 FP32: tile 45.7 us, march
-// 35.7; 512 x 512: 14.3 and 16.5; thermal 16-bit 1024 x 1024: 92 and 65), and
+// whichever those figures put first (800 x 800 FP32: tile 29.4 us, march
+// 21.5; 384 x 512: 11.5 and 11.1, taken as equal; thermal 16-bit 600 x 600:
+// 38.7 and 29.4, 320 x 320: 13.6 and 13.7), and
 // on grids they do not serve the scalar march once its strips fill the GPU,
 // else the scalar tile.
 int resolved_kernel(const lb_grid* G) {
@@ -266,9 +267,9 @@ cudaError_t launch_fv_step(lb_grid* G) {
 // Whether lb_step_fv runs the two-launch step of k_fv_phase.cu: FP64 grids
 // of every size (the fused kernels recompute on the scarce FP64 pipe), and
 // x-periodic FP32-math grids up to 128 cells per SM (thermal: 64), where the fused tile
-// leaves most SMs idle: 128 x 128 FP32 takes 4.4 us a step against 6.1,
-// 192 x 192 8.1 against 6.3; thermal 96 x 96 4.9 against 9.1, 128 x 128 8.9
-// against 9.1.  Its kernels address a pair of planes with 32-bit offsets.
+// leaves most SMs idle: 128 x 128 FP32 takes 5.0 us a step against 5.5,
+// 150 x 150 7.0 against 5.4; thermal 96 x 96 5.4 against 7.0, 110 x 110 9.2
+// against 7.1.  Its kernels address a pair of planes with 32-bit offsets.
 bool phase_applies(const lb_grid* G) {
     if (G->fv_scheme != LB_FV_HEUN || has_density_axis(G)) return false;
     const bool f64 = G->prec == Prec::F64;
@@ -449,6 +450,18 @@ lb_status run_steps(lb_grid* G, int nsteps, F one) {
 }  // namespace
 
 namespace lbgb {
+// A served request leaves the batched paired tiles for launches of its own
+// where the block march is faster than the request's share of full tile
+// waves: thermal grids from about 512 x 512 (600 x 600, 16-bit: 29.5 us a
+// step against 31.8), flow grids from about 450 x 450 (600 x 600, FP32: 13.4
+// against 15.4).  Both kernels give the same bits.  160 requests of 64 x 64 to
+// 1024 x 1024 queued at once, 16-bit: 9.4 -> 12.4 GLUPS, p99 2.33 -> 1.77 s.
+bool march_served(const lb_grid* G) {
+    const double wave = G->d.thermal ? 6.7 : 6.5 / 2;
+    const long long tiles = (long long)((G->nx + 31) / 32) * ((G->ny + 15) / 16);
+    return pair_ok(G) && march_plan(G, 0).us * G->sms < wave * (double)tiles;
+}
+
 // Mass and (thermal grids) Nusselt numbers from one reduction: the figures
 // lb_conservation and lb_nusselt would give, and their status.
 lb_status final_figures(lb_grid* G, double* mass, double* nu_vol, double* nu_bot, double* nu_top) {

@@ -228,6 +228,8 @@ inline StepArgs<R> step_args(const lb_grid* G, double dt) {
     return A;
 }
 
+// whether a served request steps on the block march (lb_abi.cu)
+bool march_served(const lb_grid* G);
 // the closing figures of a served request (lb_abi.cu)
 lb_status final_figures(lb_grid* G, double* mass, double* nu_vol, double* nu_bot, double* nu_top);
 

@@ -35,6 +35,7 @@ struct Active {
     int done = 0;
     double t_submit = 0, t_admit = 0;
     size_t bytes = 0;
+    bool march = false;  // steps on the block march while the batch is of paired tiles
 };
 
 struct Pending {
@@ -268,8 +269,8 @@ lb_status lb_server_pump(lb_server* S, int* n_active, int* n_pending) {
         lb_status st = lb_create_grid(&d, &a.grid);
         if (st == LB_OK) st = lb_init(a.grid, &p.req.params, &p.req.init);
         if (st == LB_OK) {
-            // the batched kernels use the tile decomposition
-            a.grid->fv_kernel = LB_FV_TILE;
+            a.march = march_served(a.grid);
+            a.grid->fv_kernel = a.march ? LB_FV_PAIR : LB_FV_TILE;
             a.t_admit = S->now();
             S->used += need;
             S->active.push_back(a);
@@ -330,17 +331,20 @@ lb_status lb_server_pump(lb_server* S, int* n_active, int* n_pending) {
                 if (run[order[j]] && j > 0) sum += t;
             }
         }
+        // large requests take the block march, the others the batched tiles
+        const bool split = paired(S);
+        auto marches = [&](const Active& a) { return split && a.march; };
         int ntiles = 0;
         for (size_t i = 0; i < S->active.size(); ++i)
-            if (run[i]) ntiles += tiles_of(S->active[i]);
-        lb_status st = ensure_capacity(S, (int)S->active.size(), ntiles);
+            if (run[i] && !marches(S->active[i])) ntiles += tiles_of(S->active[i]);
+        lb_status st = ensure_capacity(S, (int)S->active.size(), ntiles > 0 ? ntiles : 1);
         if (st != LB_OK) return st;
         int b = 0;
         for (int i = 0; i < (int)S->active.size(); ++i) {
             const Active& a = S->active[i];
             if (S->prec == Prec::F64) fill_req<double>(S, i, a);
             else fill_req<float>(S, i, a);
-            if (!run[i]) continue;
+            if (!run[i] || marches(a)) continue;
             const int nbx = (a.req.grid.nx + tx - 1) / tx, nby = (a.req.grid.ny + ty - 1) / ty;
             for (int y = 0; y < nby; ++y)
                 for (int x = 0; x < nbx; ++x) S->h_tiles[b++] = make_int4(i, x, y, 0);
@@ -354,8 +358,16 @@ lb_status lb_server_pump(lb_server* S, int* n_active, int* n_pending) {
         if (ue == cudaSuccess)
             ue = cudaMemcpyAsync(S->d_ntiles, S->h_ntiles, sizeof(int), cudaMemcpyHostToDevice, S->stream);
         if (ue != cudaSuccess) return fail(LB_ERR_CUDA, std::string("server table upload: ") + cudaGetErrorString(ue));
-        st = run_batch(S);
-        if (st != LB_OK) return st;
+        if (ntiles > 0) {
+            st = run_batch(S);
+            if (st != LB_OK) return st;
+        }
+        for (size_t i = 0; i < S->active.size(); ++i) {
+            Active& a = S->active[i];
+            if (!run[i] || !marches(a)) continue;
+            st = lb_step_fv(a.grid, a.remaining < S->K ? a.remaining : S->K);
+            if (st != LB_OK) return st;
+        }
         cudaError_t e = cudaStreamSynchronize(S->stream);
         if (e != cudaSuccess) return fail(LB_ERR_CUDA, std::string("server step: ") + cudaGetErrorString(e));
         // 3. bookkeeping and retirement
@@ -368,7 +380,7 @@ lb_status lb_server_pump(lb_server* S, int* n_active, int* n_pending) {
             const int taken = a.remaining < S->K ? a.remaining : S->K;
             a.remaining -= taken;
             a.done += taken;
-            a.grid->cur = (a.grid->cur + taken) & 1;
+            if (!marches(a)) a.grid->cur = (a.grid->cur + taken) & 1;  // lb_step_fv keeps its own
             if (a.remaining == 0) {
                 retire(S, a, LB_OK);
                 S->active.erase(S->active.begin() + i);

@@ -343,8 +343,11 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
     const unsigned cid = in ? id : 0;
     const int y = (int)(cid / (unsigned)A.nx), x = (int)(cid - (unsigned)y * (unsigned)A.nx);
     const unsigned c = (unsigned)y * A.pitch + x;
-    const unsigned pb = (unsigned)A.plane;  // elements
-    const unsigned own = (unsigned)i * pb + c, refl = (unsigned)(i - a + b) * pb + c;
+    // the lower plane of the pair a, inv(a) in 64 bits (18 planes can pass 2^32
+    // elements), the rest in 32: phase_applies bounds three planes
+    const size_t lo = (size_t)(i - a + (b < a ? b : a)) * (size_t)A.plane;
+    const unsigned two = 2u * (unsigned)A.plane;  // from one plane of the pair to the other
+    const unsigned own = c + (b < a ? two : 0u), refl = c + (b < a ? 0u : two);
     unsigned ox[4], oy[4], gx = 0, gy = 0;  // node offsets (elements); ghost flags of the four nodes
     Quick<R> kx, ky;
     auto line = [&](int pos, int n, int bc, unsigned stride, int v, unsigned* o, unsigned& g) {
@@ -383,7 +386,9 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
     }
     dependency_wait(P.early);
 
-    const R* H = CORR ? P.hs : P.h;
+    const R* H = (CORR ? P.hs : P.h) + lo;
+    R* hout = (CORR ? P.h : P.hs) + lo;
+    R* B = P.b + lo;
     R hx[4], hy[4];
     if (vx != 0) {
 #pragma unroll
@@ -393,7 +398,7 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
 #pragma unroll
         for (int s = 0; s < 4; ++s) hy[s] = H[oy[s]];
     }
-    const R fc = P.b[own];
+    const R fc = B[own];
     R v = 0;
     if (vx != 0) v = kx.x(hx, vx);
     if (vy != 0) {
@@ -407,10 +412,10 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
     R d;
     if constexpr (CORR) {
         d = mad(-A.hf, v, fc);
-        if (in) Store<S>::st(static_cast<S*>(G ? A.gout : A.fout) + (unsigned)a * pb + c, d);
+        if (in) Store<S>::st(static_cast<S*>(G ? A.gout : A.fout) + (size_t)a * A.plane + c, d);
         d = Round<S>::of(d);  // the next step starts from the stored value
     } else {
-        if (in) P.b[own] = mad(-A.hf, v, fc);
+        if (in) B[own] = mad(-A.hf, v, fc);
         d = mad(-A.dt, v, fc);
     }
     sd[i][lane] = d;
@@ -459,8 +464,8 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
         const R wr = w * sm[G ? kT + 1 : 1][lane], dm = w * sm[G ? kT : 0][lane] - d;
         const R t = k1 * dm + wr * (ev + (cu3 * kh + g));
         if (in) {
-            (CORR ? P.h : P.hs)[own] = d + t;
-            if constexpr (CORR) P.b[own] = d + R(2) * t;
+            hout[own] = d + t;
+            if constexpr (CORR) B[own] = d + R(2) * t;
         }
     } else {
         pairmath::LaneMom<TH> m;
@@ -476,8 +481,8 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
             m.T = sm[8][lane];
         }
         if (in) {
-            (CORR ? P.h : P.hs)[own] = G ? m.one_g(a, d, A.omgh) : m.one_f(a, d, A, A.omh, A.hF);
-            if constexpr (CORR) P.b[own] = G ? m.one_g(a, d, A.omg) : m.one_f(a, d, A, A.om, A.cf);
+            hout[own] = G ? m.one_g(a, d, A.omgh) : m.one_f(a, d, A, A.omh, A.hF);
+            if constexpr (CORR) B[own] = G ? m.one_g(a, d, A.omg) : m.one_f(a, d, A, A.om, A.cf);
         }
     }
 }

@@ -269,7 +269,8 @@ cudaError_t launch_fv_step(lb_grid* G) {
 // x-periodic FP32-math grids up to 128 cells per SM (thermal: 64), where the fused tile
 // leaves most SMs idle: 128 x 128 FP32 takes 5.0 us a step against 5.5,
 // 150 x 150 7.0 against 5.4; thermal 96 x 96 5.4 against 7.0, 110 x 110 9.2
-// against 7.1.  Its kernels address a pair of planes with 32-bit offsets.
+// against 7.1.  Its kernels address a pair of opposite planes, which lie two
+// planes apart, with 32-bit byte offsets: three planes stay below 2^32 bytes.
 bool phase_applies(const lb_grid* G) {
     if (G->fv_scheme != LB_FV_HEUN || has_density_axis(G)) return false;
     const bool f64 = G->prec == Prec::F64;

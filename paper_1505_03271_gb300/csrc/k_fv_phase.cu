@@ -23,7 +23,7 @@
 // FP64 step, fused tile -> this: 1 x 64 132 -> 7.3 us, 64 x 64 132 -> 8.7 us,
 // 1024 x 1024 2011 -> 654 us (0.52 -> 1.60 GLUPS).  FP32: 64 x 64 6.1 -> 3.7
 // us, thermal 64 x 64 (16-bit) 9.0 -> 4.3 us.
-#include "lb_pair.cuh"
+#include "lb_chain.cuh"
 #include "lb_phase.cuh"
 
 namespace lbgb {
@@ -214,8 +214,8 @@ __global__ void __launch_bounds__(128) k_phase_start(const PhaseArgs<R> P) {
     R d[Q], e[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) {
-        d[a] = Store<S>::ld(static_cast<const S*>(A.fin) + a * A.plane + c);
-        if constexpr (TH) e[a] = Store<S>::ld(static_cast<const S*>(A.gin) + a * A.plane + c);
+        d[a] = Chained<S>::ld(static_cast<const S*>(A.fin) + a * A.plane + c);
+        if constexpr (TH) e[a] = Chained<S>::ld(static_cast<const S*>(A.gin) + a * A.plane + c);
     }
     store_h<R, TH, true>(d, e, P, y, P.h, c);
 }

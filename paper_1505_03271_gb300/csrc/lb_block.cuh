@@ -18,6 +18,7 @@
 // threads), 512 x 512 32 -> 27 (where the march of k_fv_blocks.cu takes 23).
 #pragma once
 
+#include "lb_chain.cuh"
 #include "lb_pair.cuh"
 
 namespace lbgb {
@@ -248,18 +249,18 @@ __device__ __forceinline__ void tile_step(const StepArgs<float>& A, const int x0
         if (contiguous) {
 #pragma unroll
             for (int a = 0; a < Q; ++a) {
-                d[a] = PairIO<S>::ld(fin + a * A.plane + row + xu);
-                if constexpr (TH) e[a] = PairIO<S>::ld(gin + a * A.plane + row + xu);
+                d[a] = Chained<S>::two(fin + a * A.plane + row + xu);
+                if constexpr (TH) e[a] = Chained<S>::two(gin + a * A.plane + row + xu);
             }
         } else {
             const int gxl = ((xu % nx) + nx) % nx, gxr = ((xu + 1) % nx + nx) % nx;
 #pragma unroll
             for (int a = 0; a < Q; ++a) {
                 const S* b = fin + a * A.plane + row;
-                d[a] = mk(Store<S>::ld(b + gxl), Store<S>::ld(b + gxr));
+                d[a] = mk(Chained<S>::ld(b + gxl), Chained<S>::ld(b + gxr));
                 if constexpr (TH) {
                     const S* bg = gin + a * A.plane + row;
-                    e[a] = mk(Store<S>::ld(bg + gxl), Store<S>::ld(bg + gxr));
+                    e[a] = mk(Chained<S>::ld(bg + gxl), Chained<S>::ld(bg + gxr));
                 }
             }
         }

@@ -181,35 +181,6 @@ __device__ __forceinline__ R ref_flux(const StepArgs<R>& A, int gy, bool thermal
 
 }  // namespace lbgb
 
-namespace lbgb {
-// Steps chained by programmatic dependent launch: a kernel may be resident
-// before the previous one in its stream has finished.  It reads only constant
-// tables until chain_wait(), which returns when that kernel is complete and
-// then lets the next one in; every CTA calls it, also one with nothing to do.
-// The paired tiles use it, whose CTAs are short and stage tables first:
-// channel 256 x 512 FP32 8.1 -> 7.7 us a step, 256 x 256 5.95 -> 5.4, 16
-// served requests 16.9 -> 16.6 ms.  The block march, whose CTAs fill an SM
-// and march for longer, lost by it (1000 x 375 thermal 30.0 -> 31.5 us).
-__device__ __forceinline__ void chain_wait() {
-    cudaGridDependencySynchronize();
-    cudaTriggerProgrammaticLaunchCompletion();
-}
-template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
-}  // namespace lbgb
-
 // ---- launchers (implemented in the kernel translation units) ----
 namespace lbgb {
 enum class Prec { F64, F32, F16, BF16 };

@@ -187,8 +187,10 @@ lb_status lb_get_graph_steps(lb_grid* grid, int* n, unsigned long long* replays)
  *                f~ + Coll - dt/2 A[h^n] pass through two library-owned FP32
  *                buffers allocated on first use (same restrictions as
  *                LB_FV_PAIR); chunk 0 = 32 x 16, 16 = 16 x 16.
- * LB_FV_AUTO picks by grid size and storage (on FP64 grids and on small ones
- * the two launches of LB_FV_TILE, chunk 2).  For the marching kernels chunk = 0 lets
+ * LB_FV_AUTO picks by grid size and storage: on FP64 grids and on small ones
+ * the two launches of LB_FV_TILE, chunk 2, which pay a third launch per call,
+ * so that calls of a few steps of a small FP32, FP16 or BF16 grid take the
+ * paired tile, with the same bits.  For the marching kernels chunk = 0 lets
  * the library size the chunks to fill the GPU; for LB_FV_TILE chunk picks
  * the tile: 0 = 32 x 16, 16 = 16 x 16, 8 = 16 x 8 (smaller tiles recompute
  * more halo but suit small, latency-bound grids).  LB_ERR_ARG on an unknown
@@ -197,7 +199,8 @@ typedef enum {
     LB_FV_AUTO = 0, LB_FV_TILE = 1, LB_FV_MARCH = 2, LB_FV_PAIR = 3, LB_FV_PTILE = 4, LB_FV_SPLIT = 5
 } lb_fv_kernel;
 lb_status lb_set_fv_schedule(lb_grid* grid, int kernel, int chunk);
-/* The schedule lb_step_fv will use now (after AUTO has been resolved). */
+/* The schedule lb_step_fv will use now (after AUTO has been resolved; on small
+ * FP32, FP16 and BF16 grids that of a long call). */
 lb_status lb_get_fv_schedule(lb_grid* grid, int* kernel, int* chunk);
 
 /* FV time integration (Sec. II B 2).  LB_FV_HEUN (default) is the

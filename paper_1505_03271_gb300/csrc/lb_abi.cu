@@ -279,6 +279,23 @@ bool phase_applies(const lb_grid* G) {
     return f64 || (pair_ok(G) && (G->d.thermal ? 2LL : 1LL) * G->nx * G->ny <= 128LL * G->sms);
 }
 
+// Whether a call of n steps of such an FP32-math grid gains by the two
+// launches.  They pay a third launch per call, for h of its first state, so a
+// short call takes the paired tile (the same bits): 64 x 64 6.3 us for one
+// step against 5.2, 10.0 for two against 10.5; 139 x 139 8.8 against 5.4;
+// thermal 98 x 98 16-bit 11.2 against 6.9.  In microseconds, measured from 0.1
+// to 128 cells per SM: a step of two launches (slower at up to 8 cells per SM,
+// where a CTA has 8 cells), the start of a call, and a step of the tile.
+bool phase_pays(const lb_grid* G, int n) {
+    if (G->fv_kernel != LB_FV_AUTO || G->prec == Prec::F64) return true;
+    const bool th = G->d.thermal != 0, f16 = G->prec != Prec::F32;
+    const double c = (double)G->nx * G->ny / G->sms, over = c > 25 ? c - 25 : 0;
+    const double step = (c <= 8 ? 4.4 : th ? 4.0 : 3.7) + over * (th ? 0.043 : 0.014);
+    const double start = 2.6 + over * (th ? 0.058 : 0.005);
+    const double tile = (th ? c <= 2 ? 5.0 : 6.0 : 5.2) + (f16 ? 0.8 : 0.0);
+    return start + n * step < n * tile;
+}
+
 // The two-launch step's fields, allocated on first use; false where that is
 // not possible (no memory, or a stream capture in progress forbids it): the
 // step then takes the fused kernels.
@@ -781,7 +798,7 @@ lb_status lb_step_fv(lb_grid* G, int nsteps) {
     if (s != LB_OK) return s;
     if (nsteps < 0) return fail(LB_ERR_ARG, "nsteps must be >= 0");
     DeviceGuard dg(G->device);
-    if (nsteps > 0 && phase_applies(G) && ensure_phase(G)) {
+    if (nsteps > 0 && phase_applies(G) && phase_pays(G, nsteps) && ensure_phase(G)) {
         CK(launch_phase(G, true));
         return run_steps(G, nsteps, [G] { return launch_phase(G, false); });
     }

@@ -937,11 +937,13 @@ lb_status lb_autotune_fv(lb_grid* G, int steps) {
             return phase ? launch_phase(G, false)
                          : G->prec == Prec::F64 ? launch_fv_step<double>(G) : launch_fv_step<float>(G);
         };
-        // warm-up step, then the timed ones
-        cudaError_t e = phase ? launch_phase(G, true) : cudaSuccess;
+        // warm-up step, then the timed ones as one call of lb_step_fv takes them
+        auto start = [&] { return phase ? launch_phase(G, true) : cudaSuccess; };
+        cudaError_t e = start();
         if (e == cudaSuccess) e = one();
         G->cur ^= 1;
         cudaEventRecord(e0, G->stream);
+        if (e == cudaSuccess) e = start();
         for (int k = 0; k < steps && e == cudaSuccess; ++k) {
             e = one();
             G->cur ^= 1;

@@ -33,3 +33,12 @@ def test_one_step_calls(lbgpu, nx, ny, thermal, store, one, long):
         assert not thermal or np.array_equal(o[1], outs[0][1])
     # asked for, the two launches run at every length
     assert _launches(lb, g.set_fv_schedule(lb.LB_FV_TILE, 2), 1) == 3
+
+
+def test_autotune_times_whole_calls(lbgpu):
+    """Tuned for calls of one step, a 64 x 64 FP32 grid (three launches, 6.3 us,
+    against the paired tile's 5.2) does not take the two launches; tuned for long ones it does."""
+    lb = lbgpu
+    g = lb.Grid(64, 64, store="f32").init(kind=lb.LB_INIT_TGV, **KW)
+    assert g.autotune_fv(1) != (lb.LB_FV_TILE, 2)
+    assert g.autotune_fv(200) == (lb.LB_FV_TILE, 2)

@@ -434,9 +434,9 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
         sm[2][lane] = m.ux3;
         sm[3][lane] = m.uy3;
         if constexpr (sizeof(R) == 8) {  // formed once, not by every population's thread
-            sm[4][lane] = A.omh * m.uuneg + A.hF * m.ua3neg;
-            sm[5][lane] = A.omgh * m.uuneg;
-            sm[6][lane] = R(3) * A.hF * m.ay;
+            sm[4][lane] = m.c0_f(P);
+            sm[5][lane] = m.c0_g(P);
+            sm[6][lane] = m.cty(P);
         } else {
             sm[4][lane] = m.uuneg;
             sm[5][lane] = m.ua3neg;
@@ -449,10 +449,10 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
     }
     __syncthreads();
     if constexpr (sizeof(R) == 8) {
-        // h = d + t of population a, as CellMom forms t
+        // h = d + t of population a
         const R w = a == 0 ? wgt<R>(0) : (a <= 4 ? wgt<R>(1) : wgt<R>(5));
-        const R k1 = P.k[G], kh = P.kh[G];
-        R cu3 = vx == 0 ? R(0) : (vx > 0 ? sm[2][lane] : -sm[2][lane]);
+        R cu3 = 0;  // as in CellMom::changes: of velocities 1, 2, 5 and 6, or the negative
+        if (vx != 0) cu3 = vx > 0 ? sm[2][lane] : -sm[2][lane];
         if (vy != 0) cu3 += vy > 0 ? sm[3][lane] : -sm[3][lane];
         R ct = 0;
         if (!G) {
@@ -460,9 +460,9 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
             if (vy != 0) ct += vy > 0 ? sm[6][lane] : -sm[6][lane];
         }
         constexpr int kT = TH ? 7 : 0;  // first thermal moment
-        const R g = cu3 * kh + ct, ev = cu3 * g + sm[G ? 5 : 4][lane];
-        const R wr = w * sm[G ? kT + 1 : 1][lane], dm = w * sm[G ? kT : 0][lane] - d;
-        const R t = k1 * dm + wr * (ev + (cu3 * kh + g));
+        R S, D;
+        CellMom<TH>::parts(cu3, ct, P.kh[G], sm[G ? 5 : 4][lane], S, D);
+        const R t = CellMom<TH>::change(d, S + D, P.k[G], w, sm[G ? kT : 0][lane], sm[G ? kT + 1 : 1][lane]);
         if (in) {
             hout[own] = d + t;
             if constexpr (CORR) B[own] = d + R(2) * t;

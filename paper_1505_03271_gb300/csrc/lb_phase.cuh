@@ -42,6 +42,9 @@ template <> struct Round<__nv_bfloat16> {
 // c, as in PairMom (lb_pair.cuh, which states the algebra):
 //   f: t_a = k (w_a rp - d_a) + w_a rho (S +- D)
 //   g: the same with Td, T in place of rp, rho and no force.
+// Every rounding is written out: a call forms h of its first state in another
+// kernel than the steps before it did, and a run has the same bits however it
+// is split into calls only if no compiler chooses which products are fused.
 template <bool TH>
 struct CellMom {
     double rp, rho, ux3, uy3, ay, uuneg, ua3neg, Td, T;
@@ -56,42 +59,60 @@ struct CellMom {
             Td = ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7])) + e[8];
             const double dT0 = Td + to;
             T = dT0 + A.T0;
-            ay = A.ay + A.bg * dT0;
+            ay = __fma_rn(A.bg, dT0, A.ay);
         } else {
             ay = A.ay;
         }
-        const double ux = ((e1 + e57) - e68) * ir + A.hf * A.ax;
-        const double uy = ((e2 + e57) + e68) * ir + A.hf * ay;
-        ux3 = 3.0 * ux;
-        uy3 = 3.0 * uy;
-        uuneg = -1.5 * (ux * ux + uy * uy);
-        ua3neg = -(uy3 * ay + ux3 * A.ax);
+        const double ux = __fma_rn((e1 + e57) - e68, ir, __dmul_rn(A.hf, A.ax));
+        const double uy = __fma_rn((e2 + e57) + e68, ir, __dmul_rn(A.hf, ay));
+        ux3 = __dmul_rn(3.0, ux);
+        uy3 = __dmul_rn(3.0, uy);
+        uuneg = __dmul_rn(-1.5, __fma_rn(ux, ux, __dmul_rn(uy, uy)));
+        ua3neg = -__fma_rn(uy3, ay, __dmul_rn(ux3, A.ax));
+    }
+
+    // the parts that the populations share: C0 of f and of g, and 3 hF a_y
+    __device__ __forceinline__ double c0_f(const PhaseArgs<double>& P) const {
+        return __fma_rn(P.k[0], uuneg, __dmul_rn(P.s.hF, ua3neg));
+    }
+    __device__ __forceinline__ double c0_g(const PhaseArgs<double>& P) const { return __dmul_rn(P.k[1], uuneg); }
+    __device__ __forceinline__ double cty(const PhaseArgs<double>& P) const {
+        return __dmul_rn(__dmul_rn(3.0, P.s.hF), ay);
+    }
+
+    // Even and odd part: cu3 = 3 c.u, ct = 3 hF c.a; for -c the odd one changes
+    // sign.  t takes their sum.
+    static __device__ __forceinline__ void parts(double cu3, double ct, double kh, double C0, double& S, double& D) {
+        const double g = __fma_rn(cu3, kh, ct);
+        S = __fma_rn(cu3, g, C0);
+        D = __fma_rn(cu3, kh, g);
+    }
+    static __device__ __forceinline__ double change(double d, double sum, double k, double w, double m0, double m1) {
+        return __fma_rn(__dmul_rn(w, m1), sum, __dmul_rn(k, __fma_rn(w, m0, -d)));
     }
 
     __device__ __forceinline__ void change_f(const double* d, const PhaseArgs<double>& P, double* t) const {
-        const double cty = 3.0 * P.s.hF * ay;
-        change(d, P.k[0], P.kh[0], P.k[0] * uuneg + P.s.hF * ua3neg, P.ctx, cty, rp, rho, t);
+        changes(d, P.k[0], P.kh[0], c0_f(P), P.ctx, cty(P), rp, rho, t);
     }
     __device__ __forceinline__ void change_g(const double* e, const PhaseArgs<double>& P, double* t) const {
-        change(e, P.k[1], P.kh[1], P.k[1] * uuneg, 0.0, 0.0, Td, T, t);
+        changes(e, P.k[1], P.kh[1], c0_g(P), 0.0, 0.0, Td, T, t);
     }
 
-    __device__ __forceinline__ void change(const double* d, double k, double kh, double C0, double ctx, double cty,
-                                           double m0, double m1, double* t) const {
-        t[0] = (wgt<double>(0) * m1) * C0 + k * (wgt<double>(0) * m0 - d[0]);
+    __device__ __forceinline__ void changes(const double* d, double k, double kh, double C0, double ctx, double cty,
+                                            double m0, double m1, double* t) const {
+        t[0] = change(d[0], C0, k, wgt<double>(0), m0, m1);
         pair(d, 1, ux3, k, kh, C0, ctx, m0, m1, t);
         pair(d, 2, uy3, k, kh, C0, cty, m0, m1, t);
         pair(d, 5, ux3 + uy3, k, kh, C0, cty + ctx, m0, m1, t);
         pair(d, 6, uy3 - ux3, k, kh, C0, cty - ctx, m0, m1, t);
     }
-    // populations a and inv(a) = b
+    // populations a and inv(a)
     static __device__ __forceinline__ void pair(const double* d, int a, double cu3, double k, double kh, double C0,
                                                 double ct, double m0, double m1, double* t) {
-        const int b = inv(a);
-        const double g = cu3 * kh + ct, S = cu3 * g + C0, D = cu3 * kh + g;
-        const double w0 = wgt<double>(a) * m0, w1 = wgt<double>(a) * m1;
-        t[a] = w1 * (S + D) + k * (w0 - d[a]);
-        t[b] = w1 * (S - D) + k * (w0 - d[b]);
+        double S, D;
+        parts(cu3, ct, kh, C0, S, D);
+        t[a] = change(d[a], S + D, k, wgt<double>(a), m0, m1);
+        t[inv(a)] = change(d[inv(a)], S - D, k, wgt<double>(a), m0, m1);
     }
 };
 

@@ -167,8 +167,12 @@ lb_status lb_get_graph_steps(lb_grid* grid, int* n, unsigned long long* replays)
  *   LB_FV_TILE:  32 x 16 tiles with a 4-cell halo in both axes, three
  *                shared-memory regions per tile; chunk 2: no tiles, the
  *                predictor and the corrector as two launches over the whole
- *                grid, through three library-owned fields allocated on first
- *                use (where that fails the 32 x 16 tiles run instead);
+ *                grid, through three fields borrowed for the call from
+ *                memory the library keeps (at most 1 GiB per device) or
+ *                allocates; inside a stream capture they are the grid's own
+ *                until lb_destroy.  A call without memory for them takes the
+ *                kernels of the other schedules, which lb_get_fv_schedule
+ *                does not foresee;
  *   LB_FV_MARCH: strips of 120 columns (56 for FP64 thermal) that march up
  *                `chunk` rows each, halo only in x;
  *   LB_FV_PAIR:  strips that march up `chunk` rows (rounded up to a multiple

@@ -7,6 +7,7 @@
 #include "../../include/lb3.h"
 #include "lb3.cuh"
 #include "lb_grid.cuh"
+#include "lb_scratch.cuh"
 
 using namespace lbgb;
 
@@ -243,12 +244,12 @@ lb_status lb3_create_grid(const lb3_grid_desc* d, lb3_grid** out) {
     const int sets = d->thermal ? 2 : 1;
     cudaError_t e = cudaSuccess;
     for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
-        e = cudaMalloc(&G->f[b], pop);
-        if (e == cudaSuccess && d->thermal) e = cudaMalloc(&G->g[b], pop);
+        e = device_malloc(&G->f[b], pop);
+        if (e == cudaSuccess && d->thermal) e = device_malloc(&G->g[b], pop);
     }
     // h, h* (and hg, hg*) carry two ghost planes on each side in z; f + Coll does not
     const size_t padded = (size_t)Q3 * n[0] * n[1] * (n[2] + 4) * rsize(G->prec);
-    for (int w = 0; w < 3 * sets && e == cudaSuccess; ++w) e = cudaMalloc(&G->work[w], w % 3 == 1 ? pop : padded);
+    for (int w = 0; w < 3 * sets && e == cudaSuccess; ++w) e = device_malloc(&G->work[w], w % 3 == 1 ? pop : padded);
     for (int a = 0; a < 3 && e == cudaSuccess; ++a) {
         const std::vector<double> m = G->ax[a].metric();
         const int n1 = n[a] + 1;
@@ -273,8 +274,8 @@ lb_status lb3_create_grid(const lb3_grid_desc* d, lb3_grid** out) {
         if (e == cudaSuccess)
             e = cudaMemcpy(G->width[a], G->ax[a].d.data(), sizeof(double) * n[a], cudaMemcpyHostToDevice);
     }
-    if (e == cudaSuccess) e = cudaMalloc(&G->fields, sizeof(double) * 5 * G->N);
-    if (e == cudaSuccess) e = cudaMalloc(&G->plane, sizeof(double) * 8 * n[2]);
+    if (e == cudaSuccess) e = device_malloc((void**)&G->fields, sizeof(double) * 5 * G->N);
+    if (e == cudaSuccess) e = device_malloc((void**)&G->plane, sizeof(double) * 8 * n[2]);
     if (e == cudaSuccess) e = cudaMalloc(&G->werr, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(G->werr, 0, sizeof(int));
     if (e != cudaSuccess) return bail(e);
@@ -383,8 +384,8 @@ lb_status lb3_autotune_fv(lb3_grid* G, int steps) {
     Dev3 dg(G->device);
     const size_t bytes = (size_t)Q3 * G->N * rsize(G->prec);
     void *sf = nullptr, *sg = nullptr;
-    CK3(cudaMalloc(&sf, bytes));
-    if (G->d.thermal && cudaMalloc(&sg, bytes) != cudaSuccess) {
+    CK3(device_malloc(&sf, bytes));
+    if (G->d.thermal && device_malloc(&sg, bytes) != cudaSuccess) {
         cudaFree(sf);
         return fail3(LB_ERR_OOM, "autotune: no memory for the state copy");
     }
@@ -565,7 +566,7 @@ lb_status lb3_set_populations(lb3_grid* G, const double* f, const double* g) {
     Dev3 dg(G->device);
     double* tmp = nullptr;
     const size_t bytes = sizeof(double) * Q3 * G->N;
-    CK3(cudaMalloc(&tmp, bytes));
+    CK3(device_malloc((void**)&tmp, bytes));
     // copies and packing in order on the grid's stream
     cudaError_t e = cudaMemcpyAsync(tmp, f, bytes, cudaMemcpyHostToDevice, G->stream);
     if (e == cudaSuccess) e = launch3_pack(G->prec, tmp, G->f[G->cur], G->N, 1.0, G->stream);
@@ -586,7 +587,7 @@ lb_status lb3_get_populations(lb3_grid* G, double* f, double* g) {
     Dev3 dg(G->device);
     double* tmp = nullptr;
     const size_t bytes = sizeof(double) * Q3 * G->N;
-    CK3(cudaMalloc(&tmp, bytes));
+    CK3(device_malloc((void**)&tmp, bytes));
     cudaError_t e = cudaSuccess;
     if (f) {
         e = launch3_unpack(G->prec, G->f[G->cur], tmp, G->N, 1.0, G->stream);

@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <optional>
 #include <set>
 #include <string>
 #include <tuple>
@@ -15,6 +16,7 @@
 
 #include "lb_grid.cuh"
 #include "lb_phase.cuh"
+#include "lb_scratch.cuh"
 
 using namespace lbgb;
 
@@ -232,8 +234,8 @@ int resolved_shape(const lb_grid* G) { return G->fv_kernel == LB_FV_PTILE ? G->f
 cudaError_t ensure_split_buffers(lb_grid* G) {
     if (G->xh) return cudaSuccess;
     const size_t bytes = sizeof(float) * (G->d.thermal ? 18 : 9) * (size_t)G->plane;
-    cudaError_t e = cudaMalloc(&G->xh, bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&G->xfc, bytes);
+    cudaError_t e = device_malloc((void**)&G->xh, bytes);
+    if (e == cudaSuccess) e = device_malloc((void**)&G->xfc, bytes);
     if (e != cudaSuccess) {
         if (G->xh) cudaFree(G->xh);
         G->xh = G->xfc = nullptr;
@@ -296,24 +298,48 @@ bool phase_pays(const lb_grid* G, int n) {
     return start + n * step < n * tile;
 }
 
-// The two-launch step's fields, allocated on first use; false where that is
-// not possible (no memory, or a stream capture in progress forbids it): the
-// step then takes the fused kernels.
-bool ensure_phase(lb_grid* G) {
-    if (G->phase) return true;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(G->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return false;
+// The two-launch step's fields (216 bytes a cell on FP64 flow grids, 432 on
+// thermal ones), borrowed for a call: a grid holds none between calls.  A call
+// that is being captured into a graph gets memory of the grid's own, which
+// the graph's launches may use until lb_destroy.  Empty where there is no
+// memory: the step then takes the fused kernels.
+class PhaseFields {
+public:
+    explicit PhaseFields(lb_grid* G) : G_(G) {
+        if (G->phase) return;  // the grid's own
+        const size_t rs = G->prec == Prec::F64 ? 8 : 4;
+        const size_t bytes = 3 * rs * (G->d.thermal ? 18 : 9) * (size_t)G->plane;
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(G->stream, &cs);
+        if (e == cudaSuccess && cs == cudaStreamCaptureStatusActive) {
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // an allocation is not part of the graph
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            e = cudaMalloc(&G->phase, bytes);
+            cudaThreadExchangeStreamCaptureMode(&mode);
+        } else if (e == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
+            if (!G->borrower) scratch_join(G->device);
+            G->borrower = true;
+            e = scratch_take(&G->phase, bytes, G->device, G->stream);
+            borrowed_ = e == cudaSuccess;
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            G->phase = nullptr;
+        }
     }
-    const size_t rs = G->prec == Prec::F64 ? 8 : 4;
-    if (cudaMalloc(&G->phase, 3 * rs * (G->d.thermal ? 18 : 9) * (size_t)G->plane) != cudaSuccess) {
-        cudaGetLastError();
-        G->phase = nullptr;
-        return false;
+    ~PhaseFields() {
+        if (!borrowed_) return;
+        scratch_give(G_->phase, G_->stream);
+        G_->phase = nullptr;
     }
-    return true;
-}
+    PhaseFields(const PhaseFields&) = delete;
+    PhaseFields& operator=(const PhaseFields&) = delete;
+    explicit operator bool() const { return G_->phase != nullptr; }
+
+private:
+    lb_grid* G_;
+    bool borrowed_ = false;
+};
 
 // start: h of the present state (before the first step of a call); else one step
 template <typename R>
@@ -612,7 +638,7 @@ lb_status lb_create_grid(const lb_grid_desc* d, lb_grid** out) {
         if (d->thermal) place(&G->g[b], pop_bytes);
     }
     place((void**)&G->fields, sizeof(double) * 4 * (size_t)G->nx * G->ny);
-    cudaError_t e = cudaMalloc(&G->arena, total);
+    cudaError_t e = device_malloc(&G->arena, total);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete G;
@@ -634,6 +660,7 @@ lb_status lb_destroy(lb_grid* G) {
     if (!G) return LB_OK;
     DeviceGuard dg(G->device);
     cudaStreamSynchronize(G->stream);
+    if (G->borrower) scratch_leave(G->device);
     release(G);
     delete G;
     return LB_OK;
@@ -798,9 +825,12 @@ lb_status lb_step_fv(lb_grid* G, int nsteps) {
     if (s != LB_OK) return s;
     if (nsteps < 0) return fail(LB_ERR_ARG, "nsteps must be >= 0");
     DeviceGuard dg(G->device);
-    if (nsteps > 0 && phase_applies(G) && phase_pays(G, nsteps) && ensure_phase(G)) {
-        CK(launch_phase(G, true));
-        return run_steps(G, nsteps, [G] { return launch_phase(G, false); });
+    if (nsteps > 0 && phase_applies(G) && phase_pays(G, nsteps)) {
+        const PhaseFields fields(G);
+        if (fields) {
+            CK(launch_phase(G, true));
+            return run_steps(G, nsteps, [G] { return launch_phase(G, false); });
+        }
     }
     return run_steps(G, nsteps,
                      [G] { return G->prec == Prec::F64 ? launch_fv_step<double>(G) : launch_fv_step<float>(G); });
@@ -890,8 +920,8 @@ lb_status lb_autotune_fv(lb_grid* G, int steps) {
     DeviceGuard dg(G->device);
     const size_t bytes = (size_t)Q * G->plane * elem_size(G->d.store);
     void *sf = nullptr, *sg = nullptr;
-    CK(cudaMalloc(&sf, bytes));
-    if (G->d.thermal && cudaMalloc(&sg, bytes) != cudaSuccess) {
+    CK(device_malloc(&sf, bytes));
+    if (G->d.thermal && device_malloc(&sg, bytes) != cudaSuccess) {
         cudaFree(sf);
         return fail(LB_ERR_OOM, "autotune: no memory for the state copy");
     }
@@ -911,7 +941,6 @@ lb_status lb_autotune_fv(lb_grid* G, int steps) {
             cands.push_back({LB_FV_SPLIT, 16});
         }
     }
-    const bool had_phase = G->phase != nullptr;
     cands.push_back({LB_FV_TILE, 2});
     for (int kern : {(int)LB_FV_MARCH, (int)LB_FV_PAIR}) {
         if (kern == LB_FV_PAIR && !pair_ok(G)) continue;
@@ -932,7 +961,12 @@ lb_status lb_autotune_fv(lb_grid* G, int steps) {
         G->fv_chunk = c.second;
         G->cur = cur0;
         const bool phase = c == std::make_pair((int)LB_FV_TILE, 2);
-        if (phase && !(phase_applies(G) && ensure_phase(G))) continue;
+        if (phase && !phase_applies(G)) continue;
+        std::optional<PhaseFields> fields;
+        if (phase) {
+            fields.emplace(G);
+            if (!*fields) continue;
+        }
         auto one = [&] {
             return phase ? launch_phase(G, false)
                          : G->prec == Prec::F64 ? launch_fv_step<double>(G) : launch_fv_step<float>(G);
@@ -970,10 +1004,6 @@ lb_status lb_autotune_fv(lb_grid* G, int steps) {
     cudaEventDestroy(e1);
     cudaFree(sf);
     if (sg) cudaFree(sg);
-    if (!had_phase && G->phase && (st != LB_OK || pick != std::make_pair((int)LB_FV_TILE, 2))) {
-        cudaFree(G->phase);
-        G->phase = nullptr;
-    }
     if (st != LB_OK) {
         G->fv_kernel = k0;
         G->fv_chunk = c0;
@@ -1059,7 +1089,7 @@ lb_status lb_set_populations(lb_grid* G, const double* f, const double* g) {
     DeviceGuard dg(G->device);
     const size_t n = (size_t)Q * G->nx * G->ny;
     double* tmp = nullptr;
-    CK(cudaMalloc(&tmp, sizeof(double) * n));
+    CK(device_malloc((void**)&tmp, sizeof(double) * n));
     lb_status st = LB_OK;
     const double* srcs[2] = {f, g};
     void* dsts[2] = {G->f[G->cur], G->g[G->cur]};
@@ -1089,7 +1119,7 @@ lb_status lb_get_window(lb_grid* G, int x0, int y0, int w, int h, double* f, dou
     y0 = ((y0 % G->ny) + G->ny) % G->ny;
     const size_t n = (size_t)Q * w * h;
     double* tmp = nullptr;
-    CK(cudaMalloc(&tmp, sizeof(double) * n));
+    CK(device_malloc((void**)&tmp, sizeof(double) * n));
     lb_status st = LB_OK;
     double* dsts[2] = {f, g};
     const void* srcs[2] = {G->f[G->cur], G->g[G->cur]};

@@ -155,7 +155,8 @@ struct lb_grid {
     float* xh = nullptr;        // split schedule: h*, [NQ][ny][pitch] FP32 (allocated on first use)
     float* xfc = nullptr;       // split schedule: f~ + Coll - dt/2 A[h^n]
     void* fold[2] = {nullptr, nullptr};  // Axis::cell_weights of x and y, compute precision
-    void* phase = nullptr;      // two-launch step: h, h*, b, each [NQ][ny][pitch] (allocated on first use)
+    void* phase = nullptr;      // two-launch step: h, h*, b, each [NQ][ny][pitch] (a call's; the grid's own once captured)
+    bool borrower = false;      // has borrowed scratch memory (lb_scratch.cuh)
     double* fields = nullptr;   // [4][ny][nx] staging for init/moments
     double* partial = nullptr;  // reduction partials
     double* red = nullptr;      // reduction totals

@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "lb_grid.cuh"
+#include "lb_scratch.cuh"
 
 using namespace lbgb;
 
@@ -108,7 +109,8 @@ lb_status ensure_capacity(lb_server* S, int nreq, int ntiles) {
     S->h_tiles = nullptr;
     ++S->table_gen;  // the old tables are gone: any captured graph is stale
     const size_t rs = req_size(S->prec);
-    if (cudaMalloc(&S->d_reqs, rs * cr) != cudaSuccess || cudaMalloc((void**)&S->d_tiles, sizeof(int4) * ct) != cudaSuccess ||
+    if (device_malloc(&S->d_reqs, rs * cr) != cudaSuccess ||
+        device_malloc((void**)&S->d_tiles, sizeof(int4) * ct) != cudaSuccess ||
         cudaMallocHost(&S->h_reqs, rs * cr) != cudaSuccess ||
         cudaMallocHost((void**)&S->h_tiles, sizeof(int4) * ct) != cudaSuccess) {
         cudaGetLastError();
@@ -257,6 +259,9 @@ lb_status lb_server_pump(lb_server* S, int* n_active, int* n_pending) {
         const size_t need = grid_bytes(p.req.grid);
         size_t free_b = 0, total_b = 0;
         cudaError_t me = cudaMemGetInfo(&free_b, &total_b);
+        if (me == cudaSuccess && S->used + need <= S->budget && need + (64u << 20) > free_b &&
+            scratch_reclaim(S->device))
+            me = cudaMemGetInfo(&free_b, &total_b);
         if (me != cudaSuccess) return fail(LB_ERR_CUDA, std::string("server admission: ") + cudaGetErrorString(me));
         if (S->used + need > S->budget || need + (64u << 20) > free_b) break;
         Active a;

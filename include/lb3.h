@@ -112,9 +112,10 @@ lb_status lb3_set_fv_staged_shape(lb3_grid* grid, int rows, int planes, int ahea
 /* The shape the staged passes use (defaults resolved for this grid). */
 lb_status lb3_get_fv_staged_shape(lb3_grid* grid, int* rows, int* planes, int* ahead);
 /* Times the flux schedules on the grid's current state (one warm-up step and
- * `steps` timed steps each, CUDA events on the grid's stream), keeps the
- * fastest and restores the state bit for bit.  Candidates: the plain passes,
- * and where the grid allows them the staged passes with rows per tile
+ * one timed call of `steps` steps each, CUDA events on the grid's stream),
+ * keeps the fastest and restores the state bit for bit.  Candidates: the two
+ * passes of LB3_FV_AUTO on grids that get them, the plain passes, and where the
+ * grid allows them the staged passes with rows per tile
  * {default, default / 2}, planes per CTA {16, 32} and planes ahead {2, 3}.
  * LB_ERR_ARG for steps < 1; LB_ERR_OOM without room for a copy of the
  * state; LB_ERR_TIMEOUT (grid poisoned) if a timed step's wait ran out. */

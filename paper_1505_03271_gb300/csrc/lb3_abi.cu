@@ -362,18 +362,25 @@ static cudaError_t fv3_step(lb3_grid* G) {
     return e;
 }
 
+// nsteps steps as one call of lb3_step_fv takes them
+static cudaError_t fv3_steps(lb3_grid* G, int nsteps) {
+    cudaError_t e = cudaSuccess;
+    if (passes3(G) && nsteps > 0) {
+        Args3<float> A = args3<float>(G, false);
+        e = launch3_fv_passes(G->d.thermal != 0, &A, nsteps, G->stream);
+        if (e == cudaSuccess) G->cur ^= 1;  // only the last step writes the state
+        return e;
+    }
+    for (int k = 0; k < nsteps && e == cudaSuccess; ++k) e = fv3_step(G);
+    return e;
+}
+
 lb_status lb3_step_fv(lb3_grid* G, int nsteps) {
     lb_status s = ready3(G);
     if (s != LB_OK) return s;
     if (nsteps < 0) return fail3(LB_ERR_ARG, "nsteps must be >= 0");
     Dev3 dg(G->device);
-    if (passes3(G) && nsteps > 0) {
-        Args3<float> A = args3<float>(G, false);
-        CK3(launch3_fv_passes(G->d.thermal != 0, &A, nsteps, G->stream));
-        G->cur ^= 1;  // only the last step writes the state
-        return LB_OK;
-    }
-    for (int k = 0; k < nsteps; ++k) CK3(fv3_step(G));
+    CK3(fv3_steps(G, nsteps));
     return LB_OK;
 }
 
@@ -395,7 +402,8 @@ lb_status lb3_autotune_fv(lb3_grid* G, int steps) {
     struct Cand {
         int sched, rows, planes, ahead;
     };
-    std::vector<Cand> cands = {{LB3_FV_PLAIN, 0, 0, 0}};
+    // AUTO first: its two passes are no other candidate's, and without them it is a staged one
+    std::vector<Cand> cands = {{LB3_FV_AUTO, 0, 0, 0}, {LB3_FV_PLAIN, 0, 0, 0}};
     if (staged_ok3(G)) {
         int ty = 0, kc = 0, ah = 0;
         adv3_staged_resolve(G->n, G->prec, &ty, &kc, &ah);
@@ -409,7 +417,7 @@ lb_status lb3_autotune_fv(lb3_grid* G, int steps) {
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     float best = 1e30f;
-    Cand pick = cands[0];
+    Cand pick = cands[1];
     lb_status st = LB_OK;
     for (const Cand& c : cands) {
         G->fv_sched = c.sched;
@@ -417,9 +425,10 @@ lb_status lb3_autotune_fv(lb3_grid* G, int steps) {
         G->sshape[1] = c.planes;
         G->sshape[2] = c.ahead;
         G->cur = cur0;
-        cudaError_t e = fv3_step(G);  // warm-up, then the timed steps
+        if (c.sched == LB3_FV_AUTO && !passes3(G)) continue;
+        cudaError_t e = fv3_steps(G, 1);  // warm-up, then the timed steps
         cudaEventRecord(e0, G->stream);
-        for (int k = 0; k < steps && e == cudaSuccess; ++k) e = fv3_step(G);
+        if (e == cudaSuccess) e = fv3_steps(G, steps);
         cudaEventRecord(e1, G->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         if (e != cudaSuccess) {

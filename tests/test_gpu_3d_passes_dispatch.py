@@ -40,3 +40,18 @@ def test_autotune_keeps_two_passes(lbgpu):
         g.close()
     for a, b in zip(*outs):
         assert np.array_equal(a, b)
+
+
+def test_one_step_calls_of_larger_thermal_grids(lbgpu):
+    """Thermal 64 x 64 x 32: one step in four passes, more in two each, with the
+    bits of one call."""
+    lb = lbgpu
+    kw = dict(tau=0.2, tau_g=0.2, dt=0.2, beta=1e-2, grav=1.0, T0=1.0, T_bot=1.5, T_top=0.5)
+    outs = []
+    for calls, launches in (([1, 1, 2], [4, 4, 5]), ([4], [9])):
+        g = lb.Grid3(64, 64, 32, bcz=1, thermal=True).init(**kw, kind=lb.LB_INIT_RB, amp=1e-2, seed=11)
+        assert [_launches(lb, g, n) for n in calls] == launches
+        outs.append(g.get_pops())
+        g.close()
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)

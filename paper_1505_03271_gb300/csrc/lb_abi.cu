@@ -7,7 +7,9 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <optional>
 #include <set>
 #include <string>
@@ -93,6 +95,27 @@ struct DeviceGuard {
     ~DeviceGuard() {
         if (prev >= 0) cudaSetDevice(prev);
     }
+};
+
+// Host image of the tables from `first` up to `end` in a grid's arena, filled
+// by the pointers they have on the device and sent by one copy.
+class HostTables {
+public:
+    HostTables(void* first, const void* end)
+        : first_(static_cast<unsigned char*>(first)), buf_(static_cast<const unsigned char*>(end) - first_) {}
+    template <typename T>
+    T* at(const void* p) {
+        return reinterpret_cast<T*>(buf_.data() + (static_cast<const unsigned char*>(p) - first_));
+    }
+    void put(const void* p, const std::vector<double>& v, bool f32) {
+        if (f32) std::copy(v.begin(), v.end(), at<float>(p));
+        else std::copy(v.begin(), v.end(), at<double>(p));
+    }
+    cudaError_t upload() const { return cudaMemcpy(first_, buf_.data(), buf_.size(), cudaMemcpyHostToDevice); }
+
+private:
+    unsigned char* first_;
+    std::vector<unsigned char> buf_;
 };
 
 AuxArgs aux_args(const lb_grid* G) {
@@ -526,7 +549,7 @@ const char* lb_last_error(void) { return g_err.c_str(); }
 
 unsigned long long lb_kernel_launches(void) { return g_launches.load(); }
 
-lb_status lb_create_grid(const lb_grid_desc* d, lb_grid** out) {
+static lb_status create_grid(const lb_grid_desc* d, lb_grid** out) {
     if (!d || !out) return fail(LB_ERR_ARG, "NULL description or output");
     if (d->nx < 1 || d->ny < 1) return fail(LB_ERR_ARG, "nx, ny must be >= 1 (got %d, %d)", d->nx, d->ny);
     if ((long long)d->nx * d->ny > (1LL << 31))
@@ -548,13 +571,14 @@ lb_status lb_create_grid(const lb_grid_desc* d, lb_grid** out) {
         if ((sp == LB_AXIS_TANH || sp == LB_AXIS_SINH) && !(st > 0)) return fail(LB_ERR_ARG, "stretch must be > 0");
         if (sp == LB_AXIS_SINH && (n % 2)) return fail(LB_ERR_ARG, "sinh spacing needs an even cell count");
     }
-    lb_grid* G = new lb_grid();
-    G->d = *d;
-    G->nx = d->nx;
-    G->ny = d->ny;
-    G->pitch = ((d->nx + 31) / 32) * 32;
-    G->plane = (long long)G->pitch * d->ny;
-    G->prec = prec_of(d->store);
+    struct Drop {
+        void operator()(lb_grid* g) const {
+            release(g);
+            delete g;
+        }
+    };
+    std::unique_ptr<lb_grid, Drop> G(new lb_grid());
+    set_sizes(*G, *d);
     G->stream = static_cast<cudaStream_t>(d->cuda_stream);
     G->ax = make_axis(d->nx, d->lx, d->sx, d->stretch_x, d->bcx);
     G->ay = make_axis(d->ny, d->ly, d->sy, d->stretch_y, d->bcy);
@@ -564,96 +588,70 @@ lb_status lb_create_grid(const lb_grid_desc* d, lb_grid** out) {
     for (int k = 0; k < 2; ++k) {
         const Axis& a = k ? G->ay : G->ax;
         for (double v : a.d)
-            if (!(v > 0)) {
-                delete G;
-                return fail(LB_ERR_ARG, "degenerate cell width on axis %c", k ? 'y' : 'x');
-            }
+            if (!(v > 0)) return fail(LB_ERR_ARG, "degenerate cell width on axis %c", k ? 'y' : 'x');
     }
     cudaGetDevice(&G->device);
     cudaDeviceGetAttribute(&G->sms, cudaDevAttrMultiProcessorCount, G->device);
     if (G->sms <= 0) G->sms = 152;
-    const size_t pop_bytes = (size_t)Q * G->plane * elem_size(d->store);
-    const bool as_float = G->prec != Prec::F64;
-    const size_t rs = as_float ? sizeof(float) : sizeof(double);
-    G->nred = reduce_blocks(G->nx, G->ny);
-    // one allocation for everything the grid owns, the constant tables first
-    // and uploaded by one copy: creating and destroying a 128 x 128 thermal
-    // grid took 0.30 ms with an allocation and a copy apiece and takes 0.20,
-    // which a server pays for every request
-    size_t total = 0;
-    std::vector<std::pair<void**, size_t>> parts;  // where each pointer goes, and its offset
-    auto place = [&](void** p, size_t bytes) {
-        parts.emplace_back(p, total);
-        total += (bytes + 255) / 256 * 256;
-        return parts.back().second;
-    };
-    std::vector<unsigned char> tables;
-    auto table = [&](void** p, const std::vector<double>& v, bool f32) {
-        const size_t at = place(p, v.size() * (f32 ? sizeof(float) : sizeof(double)));
-        tables.resize(total);
-        if (f32) std::copy(v.begin(), v.end(), reinterpret_cast<float*>(tables.data() + at));
-        else std::copy(v.begin(), v.end(), reinterpret_cast<double*>(tables.data() + at));
-    };
-    const std::vector<double> mxv = G->ax.metric();
-    table(&G->mx, mxv, as_float);
-    table(&G->my, G->ay.metric(), as_float);
-    table(&G->fold[0], G->ax.cell_weights(as_float), as_float);
-    table(&G->fold[1], G->ay.cell_weights(as_float), as_float);
-    table((void**)&G->dxv, G->ax.d, false);
-    table((void**)&G->dyv, G->ay.d, false);
-    table((void**)&G->xc, G->ax.c, false);
-    table((void**)&G->yc, G->ay.c, false);
-    std::vector<double> tab(20 * (size_t)G->nx, 0.0);
-    if (as_float) {
-        // x data of the column pair starting at each column (the right column wraps)
-        const int nx = G->nx;
-        auto wpv = [&](int r, int k) { return mxv[r * (nx + 1) + k]; };
-        auto wmv = [&](int r, int k) { return mxv[(3 + r) * (nx + 1) + k]; };
-        for (int c = 0; c < nx; ++c) {
-            const int cr = (c + 1) % nx;
-            double* e = &tab[20 * (size_t)c];
-            for (int r = 0; r < 3; ++r) {
-                e[r] = wpv(r, c);
-                e[3 + r] = wpv(r, c + 1);
-                e[6 + r] = wpv(r, cr + 1);
-                e[9 + r] = wmv(r, c);
-                e[12 + r] = wmv(r, c + 1);
-                e[15 + r] = wmv(r, cr + 1);
-            }
-            e[18] = mxv[6 * (nx + 1) + c];
-            e[19] = mxv[6 * (nx + 1) + cr];
-        }
-    }
-    table((void**)&G->coltab, tab, true);
-    place((void**)&G->toff, sizeof(double) * G->ny);
-    place(&G->toff_r, rs * G->ny);
-    place((void**)&G->roff, sizeof(double) * G->ny);
-    place(&G->roff_r, rs * G->ny);
-    place(&G->dref_r, rs * 4 * G->ny);
-    place((void**)&G->rowtab, sizeof(float) * 20 * G->ny);
-    place((void**)&G->partial, sizeof(double) * kRed * G->nred);
-    place((void**)&G->red, sizeof(double) * kRed);
-    for (int b = 0; b < 2; ++b) {
-        place(&G->f[b], pop_bytes);
-        if (d->thermal) place(&G->g[b], pop_bytes);
-    }
-    place((void**)&G->fields, sizeof(double) * 4 * (size_t)G->nx * G->ny);
+    // one allocation for everything the grid owns: creating and destroying a
+    // 128 x 128 thermal grid took 0.30 ms with an allocation and a copy apiece
+    // and takes 0.20, which a server pays for every request.  It comes before
+    // the host tables, so that a grid the device cannot hold fails here.
+    const size_t total = grid_device_bytes(*d);
     cudaError_t e = device_malloc(&G->arena, total);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        delete G;
         return fail(e == cudaErrorMemoryAllocation ? LB_ERR_OOM : LB_ERR_CUDA, "cudaMalloc(%zu bytes): %s", total,
                     cudaGetErrorString(e));
     }
-    e = cudaMemcpy(G->arena, tables.data(), tables.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-        cudaFree(G->arena);
-        delete G;
-        return fail(LB_ERR_CUDA, "table upload: %s", cudaGetErrorString(e));
+    unsigned char* at = static_cast<unsigned char*>(G->arena);
+    grid_parts(*G, [&](void** p, size_t bytes) {
+        *p = at;
+        at += part_size(bytes);
+    });
+    const bool f32 = G->prec != Prec::F64;
+    HostTables tables(G->arena, G->toff);
+    const std::vector<double> mxv = G->ax.metric();
+    tables.put(G->mx, mxv, f32);
+    tables.put(G->my, G->ay.metric(), f32);
+    tables.put(G->fold[0], G->ax.cell_weights(f32), f32);
+    tables.put(G->fold[1], G->ay.cell_weights(f32), f32);
+    tables.put(G->dxv, G->ax.d, false);
+    tables.put(G->dyv, G->ay.d, false);
+    tables.put(G->xc, G->ax.c, false);
+    tables.put(G->yc, G->ay.c, false);
+    if (f32) {
+        // x data of the column pair starting at each column (the right column wraps)
+        const int nx = G->nx;
+        auto wpv = [&](int r, int k) { return (float)mxv[r * (size_t)(nx + 1) + k]; };
+        auto wmv = [&](int r, int k) { return (float)mxv[(3 + r) * (size_t)(nx + 1) + k]; };
+        for (int c = 0; c < nx; ++c) {
+            const int cr = (c + 1) % nx;
+            float* t = tables.at<float>(G->coltab) + 20 * (size_t)c;
+            for (int r = 0; r < 3; ++r) {
+                t[r] = wpv(r, c);
+                t[3 + r] = wpv(r, c + 1);
+                t[6 + r] = wpv(r, cr + 1);
+                t[9 + r] = wmv(r, c);
+                t[12 + r] = wmv(r, c + 1);
+                t[15 + r] = wmv(r, cr + 1);
+            }
+            t[18] = (float)mxv[6 * (size_t)(nx + 1) + c];
+            t[19] = (float)mxv[6 * (size_t)(nx + 1) + cr];
+        }
     }
-    for (const auto& p : parts) *p.first = static_cast<unsigned char*>(G->arena) + p.second;
-    *out = G;
+    e = tables.upload();
+    if (e != cudaSuccess) return fail(LB_ERR_CUDA, "table upload: %s", cudaGetErrorString(e));
+    *out = G.release();
     return LB_OK;
+}
+
+lb_status lb_create_grid(const lb_grid_desc* d, lb_grid** out) {
+    try {
+        return create_grid(d, out);
+    } catch (const std::bad_alloc&) {
+        return fail(LB_ERR_OOM, "no host memory for the grid's tables");
+    }
 }
 
 lb_status lb_destroy(lb_grid* G) {
@@ -673,7 +671,7 @@ lb_status lb_sync(lb_grid* G) {
     return LB_OK;
 }
 
-lb_status lb_init(lb_grid* G, const lb_params* p, const lb_init_desc* in) {
+static lb_status init_grid(lb_grid* G, const lb_params* p, const lb_init_desc* in) {
     if (!G || !p || !in) return fail(LB_ERR_ARG, "NULL argument");
     if (!(p->tau > 0) || !(p->dt > 0)) return fail(LB_ERR_ARG, "tau and dt must be > 0");
     if (G->d.thermal && !(p->tau_g > 0)) return fail(LB_ERR_ARG, "tau_g must be > 0 on a thermal grid");
@@ -727,40 +725,31 @@ lb_status lb_init(lb_grid* G, const lb_params* p, const lb_init_desc* in) {
                 for (int j = 0; j < ny; ++j) dref[(2 * q + sgn) * ny + j] = (face(j + 1) - face(j)) / G->ay.d[j];
             }
         }
-        // the tables lie side by side in the arena, toff first: one upload
-        std::vector<unsigned char> buf(reinterpret_cast<unsigned char*>(G->rowtab) - reinterpret_cast<unsigned char*>(G->toff) +
-                                       sizeof(float) * 20 * (size_t)ny);
-        auto put = [&](const void* where, const std::vector<double>& v, bool f32) {
-            unsigned char* p = buf.data() + (static_cast<const unsigned char*>(where) - reinterpret_cast<unsigned char*>(G->toff));
-            if (f32) std::copy(v.begin(), v.end(), reinterpret_cast<float*>(p));
-            else std::copy(v.begin(), v.end(), reinterpret_cast<double*>(p));
-        };
         const bool f32 = G->prec != Prec::F64;
-        put(G->toff, to, false);
-        put(G->roff, ro, false);
-        put(G->toff_r, to, f32);
-        put(G->roff_r, ro, f32);
-        put(G->dref_r, dref, f32);
+        HostTables tables(G->toff, G->partial);
+        tables.put(G->toff, to, false);
+        tables.put(G->roff, ro, false);
+        tables.put(G->toff_r, to, f32);
+        tables.put(G->roff_r, ro, f32);
+        tables.put(G->dref_r, dref, f32);
         if (f32) {
             // per-row table of the paired kernels: one 80-byte entry per row
             const std::vector<double> my = G->ay.metric();
-            std::vector<double> tab(20 * (size_t)ny, 0.0);
             for (int j = 0; j < ny; ++j) {
-                double* e = &tab[20 * (size_t)j];
+                float* t = tables.at<float>(G->rowtab) + 20 * (size_t)j;
                 for (int q = 0; q < 3; ++q) {
-                    e[q] = my[q * (ny + 1) + j];            // c > 0, south face j
-                    e[3 + q] = my[q * (ny + 1) + j + 1];    // c > 0, north face j + 1
-                    e[6 + q] = my[(3 + q) * (ny + 1) + j];  // c < 0, south
-                    e[9 + q] = my[(3 + q) * (ny + 1) + j + 1];
+                    t[q] = (float)my[q * (size_t)(ny + 1) + j];            // c > 0, south face j
+                    t[3 + q] = (float)my[q * (size_t)(ny + 1) + j + 1];    // c > 0, north face j + 1
+                    t[6 + q] = (float)my[(3 + q) * (size_t)(ny + 1) + j];  // c < 0, south
+                    t[9 + q] = (float)my[(3 + q) * (size_t)(ny + 1) + j + 1];
                 }
-                e[12] = my[6 * (ny + 1) + j];
-                e[13] = ro[j];
-                e[14] = to[j];
-                for (int q = 0; q < 4; ++q) e[15 + q] = dref[q * ny + j];
+                t[12] = (float)my[6 * (size_t)(ny + 1) + j];
+                t[13] = (float)ro[j];
+                t[14] = (float)to[j];
+                for (int q = 0; q < 4; ++q) t[15 + q] = (float)dref[q * (size_t)ny + j];
             }
-            put(G->rowtab, tab, true);
         }
-        CK(cudaMemcpy(G->toff, buf.data(), buf.size(), cudaMemcpyHostToDevice));
+        CK(tables.upload());
     }
     InitArgs a{};
     a.f = G->f[0];
@@ -818,6 +807,14 @@ lb_status lb_init(lb_grid* G, const lb_params* p, const lb_init_desc* in) {
     G->poisoned = false;
     G->cur = 0;
     return LB_OK;
+}
+
+lb_status lb_init(lb_grid* G, const lb_params* p, const lb_init_desc* in) {
+    try {
+        return init_grid(G, p, in);
+    } catch (const std::bad_alloc&) {
+        return fail(LB_ERR_OOM, "no host memory for the grid's tables");
+    }
 }
 
 lb_status lb_step_fv(lb_grid* G, int nsteps) {

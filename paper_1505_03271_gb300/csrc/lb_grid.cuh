@@ -174,6 +174,60 @@ struct lb_grid {
 
 namespace lbgb {
 
+inline void set_sizes(lb_grid& G, const lb_grid_desc& d) {
+    G.d = d;
+    G.nx = d.nx;
+    G.ny = d.ny;
+    G.pitch = (int)(((long long)d.nx + 31) / 32 * 32);
+    G.plane = (long long)G.pitch * d.ny;
+    G.prec = prec_of(d.store);
+    G.nred = reduce_blocks(d.nx, d.ny);
+}
+
+// What a grid owns, in the order of its one allocation: part(pointer, bytes)
+// for each, every part on a 256-byte boundary.  First the constant tables, up
+// to toff, then those that lb_init fills, up to partial, then the rest.
+template <typename F>
+inline void grid_parts(lb_grid& G, F part) {
+    const bool f32 = G.prec != Prec::F64;
+    const size_t rs = f32 ? 4 : 8, nx = (size_t)G.nx, ny = (size_t)G.ny;
+    part(&G.mx, rs * (7 * nx + 6));  // Axis::metric
+    part(&G.my, rs * (7 * ny + 6));
+    part(&G.fold[0], rs * (f32 ? 16 : 8) * nx);  // Axis::cell_weights
+    part(&G.fold[1], rs * (f32 ? 16 : 8) * ny);
+    part((void**)&G.dxv, 8 * nx);
+    part((void**)&G.dyv, 8 * ny);
+    part((void**)&G.xc, 8 * nx);
+    part((void**)&G.yc, 8 * ny);
+    part((void**)&G.coltab, f32 ? 80 * nx : 0);
+    part((void**)&G.toff, 8 * ny);
+    part(&G.toff_r, rs * ny);
+    part((void**)&G.roff, 8 * ny);
+    part(&G.roff_r, rs * ny);
+    part(&G.dref_r, 4 * rs * ny);
+    part((void**)&G.rowtab, f32 ? 80 * ny : 0);
+    part((void**)&G.partial, sizeof(double) * kRed * (size_t)G.nred);
+    part((void**)&G.red, sizeof(double) * kRed);
+    const size_t pops = (size_t)Q * (size_t)G.plane * elem_size(G.d.store);
+    for (int b = 0; b < 2; ++b) {
+        part(&G.f[b], pops);
+        if (G.d.thermal) part(&G.g[b], pops);
+    }
+    part((void**)&G.fields, sizeof(double) * 4 * nx * ny);
+}
+
+inline size_t part_size(size_t bytes) { return (bytes + 255) / 256 * 256; }
+
+// Device memory of a grid (0 for sizes that lb_create_grid refuses).
+inline size_t grid_device_bytes(const lb_grid_desc& d) {
+    if (d.nx < 1 || d.ny < 1) return 0;
+    lb_grid G;
+    set_sizes(G, d);
+    size_t total = 0;
+    grid_parts(G, [&](void**, size_t bytes) { total += part_size(bytes); });
+    return total;
+}
+
 template <typename R>
 inline StepArgs<R> step_args(const lb_grid* G, double dt) {
     StepArgs<R> A{};

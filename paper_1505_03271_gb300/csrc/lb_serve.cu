@@ -44,12 +44,6 @@ struct Pending {
     double t_submit = 0;
 };
 
-size_t grid_bytes(const lb_grid_desc& d) {
-    const size_t pitch = ((size_t)d.nx + 31) / 32 * 32;
-    const size_t pops = 9 * pitch * (size_t)d.ny * elem_size(d.store) * 2 * (d.thermal ? 2 : 1);
-    return pops + 4 * sizeof(double) * (size_t)d.nx * d.ny + 64 * ((size_t)d.nx + d.ny + 64);
-}
-
 lb_status fail(lb_status s, const std::string& m) { return set_last_error(s, m.c_str()); }
 
 }  // namespace
@@ -246,7 +240,7 @@ lb_status lb_server_submit(lb_server* S, const lb_request* r) {
     if (r->grid.store != S->store || (r->grid.thermal != 0) != (S->thermal != 0))
         return fail(LB_ERR_ARG, "request storage/thermal flags differ from the server's");
     if (r->nsteps < 0) return fail(LB_ERR_ARG, "nsteps must be >= 0");
-    if (grid_bytes(r->grid) > S->budget) return fail(LB_ERR_ARG, "request larger than the server's memory budget");
+    if (grid_device_bytes(r->grid) > S->budget) return fail(LB_ERR_ARG, "request larger than the server's memory budget");
     S->pending.push_back({*r, S->now()});
     return LB_OK;
 }
@@ -256,7 +250,7 @@ lb_status lb_server_pump(lb_server* S, int* n_active, int* n_pending) {
     // 1. admission in arrival order, by budget and free device memory
     while (!S->pending.empty()) {
         const Pending& p = S->pending.front();
-        const size_t need = grid_bytes(p.req.grid);
+        const size_t need = grid_device_bytes(p.req.grid);
         size_t free_b = 0, total_b = 0;
         cudaError_t me = cudaMemGetInfo(&free_b, &total_b);
         if (me == cudaSuccess && S->used + need <= S->budget && need + (64u << 20) > free_b &&

@@ -240,13 +240,15 @@ int resolved_chunk(const lb_grid* G) {
     return ch < 32 ? 32 : ch;
 }
 
-// Shape of the scalar tile that AUTO takes for FP32 arithmetic on grids with
-// walls on x: 16 x 8 while two of them per SM cover the grid (100 x 100: 5.7
-// us a step, 9.8 at 32 x 16), else 16 x 16 (333 x 257: 12.0, 12.8 at 32 x 16
-// and 12.3 at 16 x 8).
+// Shape of the scalar tile: as asked for (32 x 16 where the two launches were,
+// on a grid they do not serve), 32 x 16 for the single-stage schemes and density
+// boundaries.  AUTO on FP32-math grids with walls on x: 16 x 8 while two of them
+// per SM cover the grid (100 x 100: 5.7 us a step, 9.8 at 32 x 16), else
+// 16 x 16 (333 x 257: 12.0, 12.8 at 32 x 16 and 12.3 at 16 x 8).
 int scalar_shape(const lb_grid* G) {
-    if (G->fv_kernel == LB_FV_TILE) return G->fv_chunk;
+    if (G->fv_kernel == LB_FV_TILE) return G->fv_chunk == 2 ? 0 : G->fv_chunk;
     if (G->fv_kernel != LB_FV_AUTO || G->prec == Prec::F64 || G->d.bcx != LB_BC_WALLS) return 0;
+    if (G->fv_scheme != LB_FV_HEUN || has_density_axis(G)) return 0;
     return (long long)((G->nx + 15) / 16) * ((G->ny + 7) / 8) <= 2LL * G->sms ? 8 : 16;
 }
 
@@ -271,7 +273,7 @@ cudaError_t launch_fv_step(lb_grid* G) {
     StepArgs<R> A = step_args<R>(G, G->p.dt);
     const bool th = G->d.thermal != 0;
     if (A.stages == 1 || has_density_axis(G))  // single-stage schemes, density boundaries: scalar tile kernel
-        return launch_fv(G->prec, th, &A, G->fv_kernel == LB_FV_TILE ? G->fv_chunk : 0, G->stream);
+        return launch_fv(G->prec, th, &A, scalar_shape(G), G->stream);
     const int k = resolved_kernel(G);
     if (k == LB_FV_SPLIT) {
         cudaError_t e = ensure_split_buffers(G);

@@ -178,7 +178,7 @@ March march_plan(const lb_grid* G, int chunk) {
             return waves(n, (long long)G->sms * (wide ? 1 : 2)) * (ch / 4 + 4) * it + 1.5;
         };
         auto take = [&](long long ch) {
-            ch = (ch + 3) / 4 * 4;
+            ch = std::min((ch + 3) / 4 * 4, 1LL << 30);  // rows and CTA counts in 32 bits
             const double us = cost(ch);
             if (us < best.us) best = {wide != 0, (int)ch, us};
         };

@@ -18,3 +18,13 @@ def test_scalar_tile_reported(lbgpu, kw, scheme, asked):
     g.step_fv(3)
     assert lb.lb_kernel_launches() - n0 == 3
     g.close()
+
+
+def test_chunk_of_the_march_stays_positive(lbgpu):
+    """Any chunk beyond the grid is the whole grid."""
+    g = lbgpu.Grid(64, 40, store="f32")
+    for chunk in (2**31 - 1, 2**31 - 8, 4096):
+        g.set_fv_schedule(lbgpu.LB_FV_PAIR, chunk)
+        assert 40 <= g.fv_schedule()[1] <= chunk
+        g.init(tau=0.3, dt=0.1, kind=lbgpu.LB_INIT_TGV, u0=0.01).step_fv(2).sync()
+    g.close()

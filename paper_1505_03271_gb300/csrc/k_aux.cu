@@ -1,6 +1,6 @@
 // k_aux.cu -- initialisation, population copy-in/out, moments and the FP64
 // reductions (conservation sums, Nusselt numbers, divergence check).
-#include "lb_internal.cuh"
+#include "lb_launch.cuh"
 
 namespace lbgb {
 

@@ -13,7 +13,7 @@
 // cells next to the wall; they are never stored in HBM.  Every population
 // is read from HBM once and written once per step (halo cells re-read from
 // L2 by neighbouring CTAs).
-#include "lb_internal.cuh"
+#include "lb_launch.cuh"
 
 namespace lbgb {
 

@@ -24,6 +24,7 @@
 // instruction issue is busy for half and the FP32 pipe for 45 %; loading A's
 // populations at the end of an iteration instead of its middle costs a fifth.
 #include "lb_block.cuh"
+#include "lb_launch.cuh"
 
 namespace lbgb {
 

@@ -15,7 +15,7 @@
 // after the write, so one barrier per row suffices.  The halo is
 // recomputed only in x: (NT)/(NT - 8) for stage A, (NT - 4)/(NT - 8) for B.
 // Each thread keeps the QUICK weights of its own two x faces in registers.
-#include "lb_internal.cuh"
+#include "lb_launch.cuh"
 
 namespace lbgb {
 

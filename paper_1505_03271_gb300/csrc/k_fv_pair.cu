@@ -6,7 +6,7 @@
 //   k_fv_split_a / _c     a tile step in two launches.
 // They serve x-periodic grids; grids with walls on x use the scalar kernels.
 #include "lb_block.cuh"
-#include "lb_pair.cuh"
+#include "lb_launch.cuh"
 
 namespace lbgb {
 

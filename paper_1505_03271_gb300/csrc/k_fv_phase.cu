@@ -24,6 +24,7 @@
 // 1024 x 1024 2011 -> 654 us (0.52 -> 1.60 GLUPS).  FP32: 64 x 64 6.1 -> 3.7
 // us, thermal 64 x 64 (16-bit) 9.0 -> 4.3 us.
 #include "lb_chain.cuh"
+#include "lb_lane.cuh"
 #include "lb_phase.cuh"
 
 namespace lbgb {

@@ -19,7 +19,7 @@
 #pragma once
 
 #include "lb_chain.cuh"
-#include "lb_pair.cuh"
+#include "lb_lane.cuh"
 
 namespace lbgb {
 namespace block {

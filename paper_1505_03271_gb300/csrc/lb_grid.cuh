@@ -5,7 +5,7 @@
 #include <cmath>
 #include <vector>
 
-#include "lb_internal.cuh"
+#include "lb_launch.cuh"
 
 namespace lbgb {
 

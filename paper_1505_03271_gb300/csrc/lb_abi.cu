@@ -243,13 +243,21 @@ int resolved_chunk(const lb_grid* G) {
 // Shape of the scalar tile: as asked for (32 x 16 where the two launches were,
 // on a grid they do not serve), 32 x 16 for the single-stage schemes and density
 // boundaries.  AUTO on FP32-math grids with walls on x: 16 x 8 while two of them
-// per SM cover the grid (100 x 100: 5.7 us a step, 9.8 at 32 x 16), else
-// 16 x 16 (333 x 257: 12.0, 12.8 at 32 x 16 and 12.3 at 16 x 8).
+// per SM cover the grid (100 x 100: 6.2 us a step, 10.3 at 32 x 16), else
+// 16 x 16, of which an SM holds three (333 x 257: 12.4, 13.3 at 32 x 16; 470 x
+// 500 22.3 and 24.2; 300 x 5000 118 and 128), except where they just pass one
+// wave and two of 32 x 16 per SM do not (460 x 300: 14.3 and 13.3), or nearly
+// fill two waves (470 x 600: 25.4 and 24.6).
 int scalar_shape(const lb_grid* G) {
     if (G->fv_kernel == LB_FV_TILE) return G->fv_chunk == 2 ? 0 : G->fv_chunk;
     if (G->fv_kernel != LB_FV_AUTO || G->prec == Prec::F64 || G->d.bcx != LB_BC_WALLS) return 0;
     if (G->fv_scheme != LB_FV_HEUN || has_density_axis(G)) return 0;
-    return (long long)((G->nx + 15) / 16) * ((G->ny + 7) / 8) <= 2LL * G->sms ? 8 : 16;
+    auto tiles = [G](int tx, int ty) { return (long long)((G->nx + tx - 1) / tx) * ((G->ny + ty - 1) / ty); };
+    const long long n8 = tiles(16, 8), n16 = tiles(16, 16), n32 = tiles(32, 16);
+    if (n8 <= 2LL * G->sms) return 8;
+    const bool one_wave = n32 <= 2LL * G->sms && n16 > 3LL * G->sms;
+    const bool two_waves = n32 <= 4LL * G->sms && 2 * n32 > 7LL * G->sms;
+    return one_wave || two_waves ? 0 : 16;
 }
 
 int resolved_shape(const lb_grid* G) { return G->fv_kernel == LB_FV_PTILE ? G->fv_chunk : tile_plan(G).shape; }

@@ -28,3 +28,21 @@ def test_chunk_of_the_march_stays_positive(lbgpu):
         assert 40 <= g.fv_schedule()[1] <= chunk
         g.init(tau=0.3, dt=0.1, kind=lbgpu.LB_INIT_TGV, u0=0.01).step_fv(2).sync()
     g.close()
+
+
+@pytest.mark.parametrize("nx,ny,shape", [(100, 100, 8), (333, 257, 16), (420, 270, 0), (460, 300, 0), (470, 330, 16),
+                                         (470, 500, 16), (470, 600, 0), (300, 1200, 16)])
+def test_default_tile_between_x_walls(lbgpu, nx, ny, shape):
+    """The tile that is fastest at each size (csrc/lb_abi.cu, scalar_shape; on
+    152 SMs), with the populations of the 32 x 16 tile to FP32 rounding."""
+    import numpy as np
+    lb = lbgpu
+    g = lb.Grid(nx, ny, bcx=1, bcy=1, store="f32")
+    outs = []
+    for sched in ((0, 0), (1, 0)):
+        g.init(tau=0.3, dt=0.05, kind=lb.LB_INIT_TGV, u0=0.02).set_fv_schedule(*sched)
+        assert g.fv_schedule() == (lb.LB_FV_TILE, 0 if sched[0] else shape)
+        outs.append(g.step_fv(3).get_pops()[0])
+    wts = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
+    assert np.abs(outs[0] - outs[1]).max() <= 2e-6 * np.abs(outs[1] - wts).max()
+    g.close()

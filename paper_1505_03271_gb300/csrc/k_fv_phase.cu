@@ -393,6 +393,12 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
     dependency_wait(P.early);
 
     const R* H = (CORR ? P.hs : P.h) + lo;
+    // formed here for the 64-bit planes (64 x 64, FP64: 8.7 -> 8.5 us a step), at
+    // its use for the 32-bit ones
+    R* const h64 = (CORR ? P.h : P.hs) + lo;
+    R* const b64 = P.b + lo;
+    auto h_out = [&]() -> R& { return (kSmall ? (CORR ? P.h : P.hs) : h64)[own]; };
+    auto b_own = [&]() -> R& { return (kSmall ? P.b : b64)[own]; };
     R hx[4], hy[4];
     if (vx != 0) {
 #pragma unroll
@@ -402,7 +408,7 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
 #pragma unroll
         for (int s = 0; s < 4; ++s) hy[s] = H[oy[s]];
     }
-    const R fc = (P.b + lo)[own];
+    const R fc = b_own();
     R v = 0;
     if (vx != 0) v = kx.x(hx, vx);
     if (vy != 0) {
@@ -420,7 +426,7 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
         if (in) Store<S>::st(dst, d);
         d = Round<S>::of(d);  // the next step starts from the stored value
     } else {
-        if (in) (P.b + lo)[own] = mad(-A.hf, v, fc);
+        if (in) b_own() = mad(-A.hf, v, fc);
         d = mad(-A.dt, v, fc);
     }
     sd[i][lane] = d;
@@ -469,8 +475,8 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
         CellMom<TH>::parts(cu3, ct, P.kh[G], sm[G ? 5 : 4][lane], S, D);
         const R t = CellMom<TH>::change(d, S + D, P.k[G], w, sm[G ? kT : 0][lane], sm[G ? kT + 1 : 1][lane]);
         if (in) {
-            ((CORR ? P.h : P.hs) + lo)[own] = d + t;
-            if constexpr (CORR) (P.b + lo)[own] = d + R(2) * t;
+            h_out() = d + t;
+            if constexpr (CORR) b_own() = d + R(2) * t;
         }
     } else {
         pairmath::LaneMom<TH> m;
@@ -486,8 +492,8 @@ __global__ void __launch_bounds__((TH ? 18 : 9) * CELLS) k_phase_pop(const Phase
             m.T = sm[8][lane];
         }
         if (in) {
-            ((CORR ? P.h : P.hs) + lo)[own] = G ? m.one_g(a, d, A.omgh) : m.one_f(a, d, A, A.omh, A.hF);
-            if constexpr (CORR) (P.b + lo)[own] = G ? m.one_g(a, d, A.omg) : m.one_f(a, d, A, A.om, A.cf);
+            h_out() = G ? m.one_g(a, d, A.omgh) : m.one_f(a, d, A, A.omh, A.hF);
+            if constexpr (CORR) b_own() = G ? m.one_g(a, d, A.omg) : m.one_f(a, d, A, A.om, A.cf);
         }
     }
 }

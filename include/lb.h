@@ -183,9 +183,7 @@ lb_status lb_get_graph_steps(lb_grid* grid, int* n, unsigned long long* replays)
  *   LB_FV_PTILE: the tiles with two columns per thread-cell and packed FP32
  *                pair arithmetic (same restrictions); chunk 0 = 32 x 16,
  *                14 = 32 x 14, 16 = 16 x 16, 512 = 32 x 16 with 512 threads
- *                per CTA, 526 = 32 x 14 with 512 threads (one pass per
- *                stage; the corrector splits each cell's populations over
- *                two threads);
+ *                per CTA, 526 = 32 x 14 with 512 threads;
  *   LB_FV_SPLIT: the paired step in two launches: collision on tile + 2 and
  *                the predictor on the tile, then the corrector; h* and
  *                f~ + Coll - dt/2 A[h^n] pass through two library-owned FP32
@@ -313,9 +311,11 @@ lb_status lb_conservation_noalloc(const float* f, const float* g, int nx, int ny
  * large enough to fill the GPU (thermal from about 512 x 512) step in
  * launches of their own on LB_FV_PAIR, which gives the same bits.  Every tile
  * is stepped by the same code whatever else is in the table, so a request's
- * result is bit-for-bit the same alone and in any batch; it is the
- * LB_FV_TILE step of lb_step_fv (equal up to FP32 rounding, since the two are
- * compiled separately). */
+ * result is bit-for-bit the same alone and in any batch.  FP32, FP16 and
+ * BF16 requests with periodic x get the bits of LB_FV_PTILE; FP64 requests,
+ * and all requests while one with walls or densities on x is active, the
+ * LB_FV_TILE step (equal up to rounding, since the two are compiled
+ * separately). */
 typedef struct lb_server lb_server;
 
 typedef struct {

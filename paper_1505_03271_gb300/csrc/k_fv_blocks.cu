@@ -110,6 +110,8 @@ __global__ void __launch_bounds__(Strip<TH, UW>::NTH, MINB)
         auto fetch = [&](int row) {
             int gy;
             if (row >= ye + 4 || !map_axis(row, ny, A.bcy, gy)) return;
+            // a plane has fewer than 2^32 elements: at most 2^31 cells in at most 65535
+            // rows (the row is a grid's y in the kernels of lb_init)
             const unsigned at = (unsigned)gy * (unsigned)A.pitch;
             if (contiguous) {
 #pragma unroll

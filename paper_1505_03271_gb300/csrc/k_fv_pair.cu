@@ -362,8 +362,8 @@ k_fv_ptile_batched(const BatchReq<float>* reqs, const int4* tiles, const int* nt
     block::tile_step<S, TH, TX, TY, NTH, TH ? 1 : 2>(A, t.y * TX, t.z * TY);
 }
 
-// Thermal tiles use 512 threads (one CTA per SM by shared memory; the
-// corrector splits f and g over two threads per pair-cell), flow tiles 256.
+// Thermal tiles use 512 threads (one CTA per SM by shared memory, a thread
+// takes f and g of a column as one unit), flow tiles 256.
 template <typename S, bool TH>
 static cudaError_t run_ptile_batched(const void* reqs, const int4* tiles, const int* ntiles, int capacity, int k,
                                      cudaStream_t s) {

@@ -4,10 +4,11 @@
 // A request is an ordinary lb_grid plus a step count.  lb_server_pump()
 //   1. admits queued requests in arrival order while their device memory
 //      fits the budget and the device's free memory (others wait),
-//   2. advances every active request by up to K steps in K launches of one
-//      batched FV kernel over a device table of (request, tile) entries; the
-//      K launches are captured once in a CUDA graph and replayed while the
-//      table's capacity is unchanged (only the table contents change),
+//   2. advances every active request by up to K steps: large ones on the block
+//      march, in launches of their own (march_served), the others in K launches
+//      of one batched FV kernel over a device table of (request, tile) entries,
+//      captured once in a CUDA graph and replayed while the table's capacity
+//      is unchanged (only the table contents change),
 //   3. retires requests that have taken all their steps: Nusselt numbers and
 //      mass are computed, the grid is freed, the result is queued.
 // Every tile is stepped by the same code whatever else is in the table, so a
